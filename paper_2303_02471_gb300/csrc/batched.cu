@@ -66,7 +66,7 @@ struct BTask {
     Ctrl *ctrl;
     int64_t hmax;          // hash_cta_max
     int64_t cap_cta;       // CTA hash table slots
-    int64_t cap_dense;     // dense values kept in shared memory
+    int64_t cap_dense;     // backward: dC entries of a column kept in shared memory
     int64_t Wmax;          // largest bitmap (words) of a product with CTA-level columns
     int64_t cap_sym;       // symbolic CTA key table slots
     const int64_t *op;     // Op of every global column
@@ -222,7 +222,7 @@ __global__ void k_bfix(BTask b, int64_t *ccp_all, int64_t total, const int64_t *
 }
 
 // ---------------------------------------------------- persistent kernels
-// Smem layout of a CTA item: [walk][table | L0 | L1 | wlist] or [walk][bm | acc].
+// Smem layout of a CTA item: [walk][table | L0 | L1 | wlist] or [walk][bm].
 struct ItemRef {
     int bin;
     int64_t idx;  // index in the bin's range
@@ -404,14 +404,10 @@ __device__ __noinline__ void bnum_cta(const BTask &b, const BProb &P, int64_t j,
     const int64_t c0 = P.Ccp[j], nn = P.Ccp[j + 1] - c0;
     if (bin == BIN_DENSE) {
         uint2 *bm = reinterpret_cast<uint2 *>(p);
-        VT *acc = reinterpret_cast<VT *>(p + al16((size_t)b.Wmax * 8));
         for (int64_t i = threadIdx.x; i < W; i += blockDim.x) bm[i] = make_uint2(0u, 0u);
         __syncthreads();
-        // double sums go to C in place (RED.F64 beats shared-memory f64
-        // atomics on GB300); float sums stay in shared memory
-        const int64_t cap = sizeof(VT) == 8 ? 0 : b.cap_dense;
-        const bool ok = num_dense_column<VT>(prob_ops<VT>(P), (int32_t)j, c0, nn, bm, W, nullptr, acc, cap, w,
-                                             s_warp, s_occ, P.Crow, static_cast<VT *>(P.Cval), []() {});
+        const bool ok = num_dense_column<VT>(prob_ops<VT>(P), (int32_t)j, c0, nn, bm, W, nullptr, w, s_warp,
+                                             s_occ, P.Crow, static_cast<VT *>(P.Cval), []() {});
         if (!ok && threadIdx.x == 0) set_error(b.ctrl, SPG_ERR_INVALID, kDetailCountMismatch + bin, j);
         return;
     }
@@ -761,7 +757,7 @@ size_t phase_smem(const spg_bplan &P, int phase, int threads, int64_t &cap_cta, 
     }
     const size_t fixed = walk + (phase == 2 ? al16((size_t)threads * 4) : 0) + al16((size_t)P.Wmax * 8);
     const size_t room = P.smem_optin > fixed ? P.smem_optin - fixed : 0;
-    cap_dense = std::min<int64_t>((int64_t)(room / w), (int64_t)P.host.maxnnz[BIN_DENSE]);
+    cap_dense = 0;
     if (phase == 2) {
         // CTA-level columns of the backward all use the dense lookup
         int64_t mx = (int64_t)P.host.maxnnz[BIN_DENSE];
@@ -770,7 +766,7 @@ size_t phase_smem(const spg_bplan &P, int phase, int threads, int64_t &cap_cta, 
         if (cta || dense) need = std::max(need, fixed + (size_t)cap_dense * w);
         return need;
     }
-    if (dense) need = std::max(need, fixed + (size_t)cap_dense * w);
+    if (dense) need = std::max(need, fixed);
     if (cta)
         need = std::max(need, walk + (P.any_f64 ? cta_table_bytes<double>(cap_cta) : cta_table_bytes<float>(cap_cta)) +
                                   al16((size_t)P.Wmax * 4) + al16((size_t)W1 * 4));

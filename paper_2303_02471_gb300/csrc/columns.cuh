@@ -267,17 +267,19 @@ __device__ __forceinline__ bool num_cta_column(const TOps<VT> &o, int32_t j, int
 // Column j by the dense SPA (Algorithm 1): flags as a bitmap (from `keep`
 // when the symbolic phase kept them, else a first product walk), prefix
 // counts, then every product is added at its row's position in the sorted
-// column, and the rows are written in ascending order.  The sums of the
-// first `cap` positions live in shared memory (s_acc), the others in place
-// in C, so the shared-memory and the L2 atomic units both take products.
+// column, in place in C (RED.F64 / RED.F32 into the L2-resident slice), and
+// the rows are written in ascending order.  Sums in shared memory were
+// measured slower in both precisions: double adds there are CAS loops, and a
+// column's float sums took the shared memory that lets four CTAs share an SM
+// (R-MAT 2^16 in float, both phases: 2.89 ms with one 1024-thread CTA
+// per SM and the sums in shared memory, 1.35 ms so).
 // bm (W uint2) is zero on entry and on return.  after_prefix() runs on
 // every thread once the flags (and `keep`) have been read.  Returns false on
 // a count mismatch.
 template <typename VT, typename AP>
 __device__ __forceinline__ bool num_dense_column(const TOps<VT> &o, int32_t j, int64_t c0, int64_t nn, uint2 *bm,
-                                                 int64_t W, const uint32_t *keep, VT *s_acc, int64_t cap,
-                                                 const WalkSmem<VT> &w, int64_t *s_warp, unsigned *s_next,
-                                                 int32_t *Crow, VT *Cval, AP &&after_prefix,
+                                                 int64_t W, const uint32_t *keep, const WalkSmem<VT> &w, int64_t *s_warp,
+                                                 unsigned *s_next, int32_t *Crow, VT *Cval, AP &&after_prefix,
                                                  int64_t *cnt_out = nullptr) {
     // the previous user of *s_next finished before the caller's last barrier
     if (threadIdx.x == 0) *s_next = (blockDim.x >> 5) * kVisitGroup;
@@ -302,36 +304,18 @@ __device__ __forceinline__ bool num_dense_column(const TOps<VT> &o, int32_t j, i
     }
     // nn <= m < 2^31: positions are 32-bit
     const int32_t n32 = (int32_t)nn;
-    // double sums always go to C in place (cap is 0 for them): a compile-time
-    // 0 drops the shared-memory path and its registers from that kernel
-    const int32_t ns = sizeof(VT) == 8 ? 0 : (int32_t)(nn < cap ? nn : cap);
     VT *gacc = Cval + c0;
     int32_t *crow = Crow + c0;
     // the extraction stages rows in the walk's scratch, free once cta_walk
     // has returned (it ends with a barrier): 20 bytes per thread
     static_assert(kVisitStage * 4 <= 32 * (16 + sizeof(float)), "visit staging exceeds the walk scratch");
     int32_t *stage = reinterpret_cast<int32_t *>(w.a0);
-    for (int32_t i = threadIdx.x; i < ns; i += blockDim.x) s_acc[i] = VT(0);
-    for (int32_t i = ns + threadIdx.x; i < n32; i += blockDim.x) gacc[i] = VT(0);
+    for (int32_t i = threadIdx.x; i < n32; i += blockDim.x) gacc[i] = VT(0);
     __syncthreads();
-    if (ns == 0) {  // every sum in C (uniform over the CTA)
-        cta_walk<true, VT, kWalkAhead>(o.Acp, o.Arow, o.Aval, o.Brow, o.Bval, o.Bcp[j], o.Bcp[j + 1], w,
-                           [&](int32_t row, VT prod) { atomicAdd(&gacc[bitmap_rank(bm, row)], prod); });
-        cta_bitmap_visit(bm, W, true, s_next, stage, [&](int32_t row) { return o.crow(row); },
-                         [&](int32_t rank, int32_t r) { crow[rank] = r; });
-    } else {
-        cta_walk<true, VT, kWalkAhead>(o.Acp, o.Arow, o.Aval, o.Brow, o.Bval, o.Bcp[j], o.Bcp[j + 1], w,
-                           [&](int32_t row, VT prod) {
-                               const int32_t r = bitmap_rank(bm, row);
-                               if (r < ns) atomicAdd(&s_acc[r], prod);
-                               else atomicAdd(&gacc[r], prod);
-                           });
-        cta_bitmap_visit(bm, W, true, s_next, stage, [&](int32_t row) { return o.crow(row); },
-                         [&](int32_t rank, int32_t r) {
-                             crow[rank] = r;
-                             if (rank < ns) gacc[rank] = s_acc[rank];
-                         });
-    }
+    cta_walk<true, VT, kWalkAhead>(o.Acp, o.Arow, o.Aval, o.Brow, o.Bval, o.Bcp[j], o.Bcp[j + 1], w,
+                                   [&](int32_t row, VT prod) { atomicAdd(&gacc[bitmap_rank(bm, row)], prod); });
+    cta_bitmap_visit(bm, W, true, s_next, stage, [&](int32_t row) { return o.crow(row); },
+                     [&](int32_t rank, int32_t r) { crow[rank] = r; });
     __syncthreads();
     return true;
 }

@@ -830,7 +830,8 @@ struct Geo {
     size_t smem = 0;       // dynamic shared memory
     int64_t slots = 0;     // table slots per CTA (CTA hash bins, global bin)
     bool bm_global = false;  // dense flags bitmap in global scratch
-    int64_t cap = 0;       // dense bin: values kept in shared memory up to this nnz
+    int64_t cap = 0;       // backward dense bin: dC kept in shared memory up to this nnz;
+                           //   CTA hash bins: 1 when the table lives in global scratch
     bool prefetch = false;   // dense bin: next column's kept flags staged by a bulk copy
 };
 

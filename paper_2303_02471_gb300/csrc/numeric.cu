@@ -13,8 +13,8 @@
 //     (kept from the symbolic phase and staged one column ahead by a bulk
 //     copy, or set again by a first walk), prefix counts turn each row into
 //     its position in the sorted column, a walk adds every product at that
-//     position (double sums in place in C, float sums in shared memory), and
-//     a pass over the flags writes the rows in order.
+//     position in place in C, and a pass over the flags writes the rows in
+//     order.
 #include "columns.cuh"
 
 namespace spg {
@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(1024, 1) k_num_cta(BinTask t, Operands o, cons
 // the current column's walk and extraction.
 template <typename VT, bool BSM>
 __global__ void __launch_bounds__(1024, 1) k_num_dense(BinTask t, Operands o, const int64_t *Ccp, int32_t *Crow,
-                                                    VT *Cval, int64_t cap, int prefetch) {
+                                                    VT *Cval, int prefetch) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int64_t s_col;
     __shared__ int64_t s_warp[32];
@@ -122,9 +122,7 @@ __global__ void __launch_bounds__(1024, 1) k_num_dense(BinTask t, Operands o, co
     const size_t o_walk = walk_smem_bytes<VT>(blockDim.x);
     uint2 *bm = BSM ? reinterpret_cast<uint2 *>(smem + o_walk)
                     : reinterpret_cast<uint2 *>(t.scratch + (size_t)blockIdx.x * t.scratch_stride);
-    VT *s_acc = reinterpret_cast<VT *>(smem + o_walk + (BSM ? (size_t)t.W * 8 : 0));
-    uint32_t *stage = reinterpret_cast<uint32_t *>(smem + o_walk + (BSM ? (size_t)t.W * 8 : 0) +
-                                                   al16((size_t)cap * sizeof(VT)));
+    uint32_t *stage = reinterpret_cast<uint32_t *>(smem + o_walk + (BSM ? (size_t)t.W * 8 : 0));
     const int64_t n_cached = t.cache_cols < t.count ? t.cache_cols : t.count;
     const unsigned stage_bytes = (unsigned)(t.W * 4);
     for (int64_t i = threadIdx.x; i < t.W; i += blockDim.x) bm[i] = make_uint2(0u, 0u);
@@ -163,8 +161,8 @@ __global__ void __launch_bounds__(1024, 1) k_num_dense(BinTask t, Operands o, co
                     bulk_load(stage, t.flag_cache + (size_t)s_col * t.W, stage_bytes, &s_bar);
             }
         };
-        const bool ok = num_dense_column<VT>(ops, j, c0, nn, bm, t.W, keep, s_acc, cap, w, s_warp, &s_chunk, Crow,
-                                             Cval, next, t.cnt_out);
+        const bool ok = num_dense_column<VT>(ops, j, c0, nn, bm, t.W, keep, w, s_warp, &s_chunk, Crow, Cval,
+                                             next, t.cnt_out);
         if (!ok && threadIdx.x == 0) set_error(t.ctrl, SPG_ERR_INVALID, kDetailCountMismatch + t.bin, j);
     }
     // a copy is in flight only after a time-out: wait for it (bounded, at
@@ -218,27 +216,15 @@ static Geo numeric_geometry_t(int bin, int64_t count, int64_t m, int threads, in
     }
     // dense
     const size_t bmb = (size_t)W * 8;
-    // shape of one CTA with t threads: its cap (values kept in shared
-    // memory), dynamic shared memory, staging of the next column's flags,
-    // and CTAs per SM
+    // shape of one CTA with t threads: dynamic shared memory, staging of the
+    // next column's flags, and CTAs per SM
     auto shape = [&](int tt, Geo &o) {
         o = g;
         o.threads = tt;
         const size_t walk = walk_smem_bytes<VT>(tt);
         o.bm_global = bmb > kBitmapSmemMax || walk + bmb > smem_optin;
         const size_t base = walk + (o.bm_global ? 0 : bmb);
-        const size_t room = smem_optin > base ? (smem_optin - base) & ~size_t(15) : 0;
-        int64_t cap = (int64_t)(room / sizeof(VT));
-        if (cap > maxnnz) cap = maxnnz;
-        // Double sums go to C in place: on GB300 a walk that adds with
-        // RED.F64 into L2-resident C takes about 1.3x the products per
-        // SM-second of one that adds with shared-memory f64 atomics (also
-        // when the first positions of a column stay in shared memory), and
-        // the extraction then copies no values.  Float sums stay in shared
-        // memory (native f32 atomics).
-        if (sizeof(VT) == 8) cap = 0;
-        o.cap = cap;
-        o.smem = base + al16((size_t)cap * sizeof(VT));
+        o.smem = base;
         int occ = occupancy(k_num_dense<VT, true>, tt, o.smem);
         // staging buffer for the next column's kept flags: bulk copies need
         // 16-byte aligned columns (W a multiple of 4); only if it costs no CTA
@@ -252,13 +238,13 @@ static Geo numeric_geometry_t(int bin, int64_t count, int64_t m, int threads, in
         }
         return occ;
     };
-    // With the double sums in C a CTA holds only the walk scratch and the
+    // With the sums in C a CTA holds only the walk scratch and the
     // flags: where four 256-thread CTAs fit an SM they beat two of 512 (more
     // CTAs overlap one another's per-column barriers; measured), else two of
     // 512, else the configured size.
     Geo g256, g512;
     int occ = 0;
-    if (sizeof(VT) == 8 && threads >= 256) {
+    if (threads >= 256) {
         const int o256 = shape(256, g256);
         const int o512 = threads >= 512 ? shape(512, g512) : 0;
         if (o256 * 256 >= o512 * 512) { g = g256; occ = o256; }
@@ -306,7 +292,7 @@ static cudaError_t launch_numeric_t(const BinTask &t, const Operands &o, const i
     } else {
         auto k = g.bm_global ? k_num_dense<VT, false> : k_num_dense<VT, true>;
         allow_smem(k, g.smem);
-        k<<<g.grid, g.threads, g.smem, s>>>(t, o, Ccp, Crow, Cval, g.cap, g.prefetch ? 1 : 0);
+        k<<<g.grid, g.threads, g.smem, s>>>(t, o, Ccp, Crow, Cval, g.prefetch ? 1 : 0);
     }
     return cudaGetLastError();
 }
