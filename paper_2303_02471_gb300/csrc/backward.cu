@@ -136,15 +136,43 @@ static Geo backward_geometry_t(int bin, int64_t count, int64_t m, int threads, i
         g.grid = (int)std::max<int64_t>(1, grid);
         return g;
     }
+    // Dense: as in the numeric phase, several CTAs per SM overlap one
+    // another's per-column barriers (backward of R-MAT 2^16 squared in
+    // double: 3.07 ms with one 1024-thread CTA per SM and a segmented scan
+    // per window, 1.51 ms now): 256 threads where that
+    // keeps as many threads resident as 512, else 512.  The CTA's share of
+    // the SM's shared memory then holds dC[:, j] of the columns it fits.
     const size_t bmb = (size_t)W * 8;
-    g.bm_global = bmb > kBitmapSmemMax || fixed + bmb > smem_optin;
-    const size_t base = fixed + (g.bm_global ? 0 : bmb);
-    const size_t room = smem_optin > base ? smem_optin - base : 0;
-    int64_t cap = (int64_t)(room / sizeof(VT));
-    if (cap > maxnnz) cap = maxnnz;
-    g.cap = cap;
-    g.smem = base + (size_t)cap * sizeof(VT);
-    int occ = occupancy(k_bwd_dense<VT, true>, g.threads, g.smem);
+    auto shape = [&](int tt, Geo &o) {
+        o = g;
+        o.threads = tt;
+        const size_t fx = walk_smem_bytes<VT>(tt) + al16((size_t)tt * 4);
+        o.bm_global = bmb > kBitmapSmemMax || fx + bmb > smem_optin;
+        o.smem = fx + (o.bm_global ? 0 : bmb);
+        int occ = occupancy(k_bwd_dense<VT, true>, tt, o.smem);
+        // flags in the per-CTA scratch: no more CTAs than it has slots for
+        if (o.bm_global) occ = (int)std::max<int64_t>(1, std::min<int64_t>(occ, scratch_ctas / sms));
+        return occ;
+    };
+    int occ = 0;
+    if (threads >= 512) {
+        Geo g256, g512;
+        const int o256 = shape(256, g256), o512 = shape(512, g512);
+        if (o256 * 256 >= o512 * 512) { g = g256; occ = o256; }
+        else { g = g512; occ = o512; }
+    } else {
+        Geo gc;
+        occ = shape(threads, gc);
+        g = gc;
+    }
+    // kSmemReserve: what the runtime and the kernel's static arrays take
+    constexpr size_t kSmemReserve = 2048;
+    const size_t share = (smem_optin / occ) & ~size_t(127);
+    g.cap = 0;
+    if (share > g.smem + kSmemReserve)
+        g.cap = std::min<int64_t>(maxnnz, (int64_t)((share - kSmemReserve - g.smem) / sizeof(VT)));
+    if (g.cap > 0 && occupancy(k_bwd_dense<VT, true>, g.threads, g.smem + (size_t)g.cap * sizeof(VT)) < occ) g.cap = 0;
+    g.smem += (size_t)g.cap * sizeof(VT);
     int64_t grid = std::min<int64_t>(count, (int64_t)occ * sms);
     if (g.bm_global) grid = std::min<int64_t>(grid, scratch_ctas);
     g.grid = (int)std::max<int64_t>(1, grid);

@@ -5,9 +5,9 @@
 // pop work items from a global counter:
 //   * a CTA item is one column of a CTA hash bin or of the dense bin;
 //   * a group item is blockDim / G columns of a warp-group bin;
-//   * in the symbolic and numeric phases, when no product has more than
-//     32 * kWarpDenseWords rows, a dense item is blockDim / 32 columns of
-//     the dense bin, one per warp.
+//   * when no product has more than 32 * kWarpDenseWords rows, a dense item
+//     is blockDim / 32 columns of the dense bin, one per warp (in the
+//     backward, CTA-level columns of up to kWarpBackwardOps products).
 // Items are ordered heaviest first (dense, then CTA bins from the largest,
 // then the group bins), the GPU form of processing columns by decreasing
 // Op_j (Section 3.1).  Per-column work is the same device code as the
@@ -53,7 +53,7 @@ struct BItems {
     int32_t order[kMaxItemBins];    // bin of each item range
     int64_t nitems;
     int nranges;
-    int dense_warp;  // dense items are groups of one column per warp
+    int dense_warp;  // dense items (backward: CTA-level items) are groups of one column per warp
 };
 
 struct BTask {
@@ -245,12 +245,41 @@ __device__ __forceinline__ ItemRef item_ref(const BItems &it, int64_t item) {
 // and warp-level synchronisation only: the column's fixed cost (clearing,
 // prefix, extraction) is small and no CTA barrier is paid per column.
 constexpr int64_t kWarpDenseWords = 1024;
+// Largest Op_j of a column that one warp takes in the backward.
+constexpr int64_t kWarpBackwardOps = 8192;
 
 // Position of row among the flagged rows of its column: the word's prefix
 // count plus the flags below it in the word.
 __device__ __forceinline__ int32_t warp_dense_rank(const uint2 *bm, int32_t row) {
     const uint2 e = bm[row >> 5];
     return (int32_t)e.y + __popc(e.x & ((1u << (row & 31)) - 1u));
+}
+
+// Prefix counts of a warp's flags into .y (each lane a contiguous run of
+// words, one warp scan); returns the number of flags.
+__device__ __forceinline__ int warp_dense_prefix(uint2 *bm, int W) {
+    const int lane = threadIdx.x & 31;
+    // an odd run per lane: the lanes' words fall in different shared-memory banks
+    const int per = ((W + 31) >> 5) | 1;
+    const int w0 = lane * per < W ? lane * per : W;
+    const int w1 = w0 + per < W ? w0 + per : W;
+    int cnt = 0;
+    for (int w = w0; w < w1; ++w) cnt += __popc(bm[w].x);
+    int incl = cnt;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += v;
+    }
+    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    int run = incl - cnt;
+    for (int w = w0; w < w1; ++w) {
+        const uint32_t x = bm[w].x;
+        bm[w].y = (uint32_t)run;
+        run += __popc(x);
+    }
+    __syncwarp();
+    return total;
 }
 
 // nnz of column j: flags set by the warp's product walk, then counted (and
@@ -301,26 +330,7 @@ __device__ __forceinline__ bool warp_dense_numeric(const TOps<VT> &o, int32_t j,
                                       [&](int32_t row, VT) { atomicOr(&bm[row >> 5].x, 1u << (row & 31)); });
     }
     __syncwarp();
-    // an odd run per lane: the lanes' words fall in different shared-memory banks
-    const int per = ((W + 31) >> 5) | 1;
-    const int w0 = lane * per < W ? lane * per : W;
-    const int w1 = w0 + per < W ? w0 + per : W;
-    int cnt = 0;
-    for (int w = w0; w < w1; ++w) cnt += __popc(bm[w].x);
-    int incl = cnt;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, d);
-        if (lane >= d) incl += v;
-    }
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    int run = incl - cnt;
-    for (int w = w0; w < w1; ++w) {
-        const uint32_t x = bm[w].x;
-        bm[w].y = (uint32_t)run;
-        run += __popc(x);
-    }
-    __syncwarp();
+    const int total = warp_dense_prefix(bm, W);
     if ((int64_t)total != nn) return false;
     VT *gacc = Cval + c0;
     int32_t *crow = Crow + c0;
@@ -340,18 +350,91 @@ __device__ __forceinline__ bool warp_dense_numeric(const TOps<VT> &o, int32_t j,
     return true;
 }
 
-// Item idx of the dense bin in warp form: warp w of the CTA takes dense
-// column idx * (warps per CTA) + w.
+// Backward of column j in one warp: C's rows set the flags, whose prefix
+// counts give the position of dC_ij; then S lanes walk each B entry's A column
+// (S the largest power of two with S times the column's entries at most 32),
+// so a * dC_ij is summed in a register and log2(S) shuffles end an entry, and
+// no search for a product's owner is needed.  Each entry of dB belongs to one
+// column: it is stored.
+template <typename VT>
+__device__ __forceinline__ void warp_dense_backward(const TOps<VT> &o, int32_t j, int64_t c0, int64_t nn,
+                                                    const int32_t *Crow, const VT *dC, uint2 *bm, int W, VT *dA,
+                                                    VT *dB) {
+    const int lane = threadIdx.x & 31;
+    for (int w = lane; w < W; w += 32) bm[w] = make_uint2(0u, 0u);
+    __syncwarp();
+    for (int64_t e = lane; e < nn; e += 32) {
+        const int32_t r = Crow[c0 + e];
+        atomicOr(&bm[r >> 5].x, 1u << (r & 31));
+    }
+    __syncwarp();
+    warp_dense_prefix(bm, W);
+    const VT *gdc = dC + c0;
+    const int64_t p0 = o.Bcp[j], p1 = o.Bcp[j + 1];
+    int S = 32;
+    while (S > 1 && (p1 - p0) * S > 32) S >>= 1;
+    const int sub = lane / S, sl = lane & (S - 1), per = 32 / S;
+    constexpr int U = 4;  // products a lane gathers at once
+    for (int64_t pb = p0; pb < p1; pb += per) {
+        const int64_t p = pb + sub;
+        int z = 0;
+        int64_t a0 = 0;
+        VT b = VT(0), acc = VT(0);
+        if (p < p1) {
+            const int32_t k = o.Brow[p];
+            a0 = o.Acp[k];
+            z = (int)(o.Acp[k + 1] - a0);
+            b = o.Bval[p];
+        }
+        for (int q0 = sl; q0 < z; q0 += U * S) {
+            int32_t row[U];
+            VT av[U], g[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int q = q0 + u * S;
+                row[u] = q < z ? o.Arow[a0 + q] : -1;
+                av[u] = q < z ? o.Aval[a0 + q] : VT(0);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) g[u] = row[u] >= 0 ? gdc[warp_dense_rank(bm, row[u])] : VT(0);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (row[u] >= 0 && dA) atomicAdd(&dA[a0 + q0 + u * S], b * g[u]);
+                acc += av[u] * g[u];
+            }
+        }
+        __syncwarp();
+        for (int d = S >> 1; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
+        if (dB && sl == 0 && p < p1) dB[p] = acc;
+    }
+}
+
+// Item idx of a bin in warp form: warp w of the CTA takes the bin's column
+// idx * (warps per CTA) + w.  The dense bin, and in the backward the CTA hash
+// bins too (every CTA-level column of the backward looks dC up by flags).
 template <int phase>
-__device__ __noinline__ void bdense_warp_item(const BTask &b, int64_t idx, unsigned char *smem) {
+__device__ __noinline__ void bdense_warp_item(const BTask &b, int bin, int64_t idx, unsigned char *smem) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int64_t k = idx * nw + warp;
-    if (k >= (int64_t)b.hist[BIN_DENSE]) return;
-    const int64_t g = b.cols[b.boff.v[BIN_DENSE] + k];
+    if (k >= (int64_t)b.hist[bin]) return;
+    const int64_t g = b.cols[b.boff.v[bin] + k];
     const int p = find_prob(b.col0s, b.nb, g);
     const BProb &P = b.prob[p];
     const int64_t j = g - P.col0;
     const int W = (int)((P.m + 31) / 32);
+    if constexpr (phase == 2) {
+        uint2 *bm = reinterpret_cast<uint2 *>(smem + (size_t)warp * al16((size_t)b.Wmax * 8));
+        const int64_t c0 = P.Ccp[j], nn = P.Ccp[j + 1] - c0;
+        if (P.dtype == SPG_F64)
+            warp_dense_backward<double>(prob_ops<double>(P), (int32_t)j, c0, nn, P.Crow,
+                                        static_cast<const double *>(P.dC), bm, W, static_cast<double *>(P.dA),
+                                        static_cast<double *>(P.dB));
+        else
+            warp_dense_backward<float>(prob_ops<float>(P), (int32_t)j, c0, nn, P.Crow,
+                                       static_cast<const float *>(P.dC), bm, W, static_cast<float *>(P.dA),
+                                       static_cast<float *>(P.dB));
+        return;
+    }
     uint32_t *keep = nullptr;
     if (b.cache && b.coff[k] + W <= b.cache_words) keep = b.cache + b.coff[k];
     if (phase == 0) {
@@ -509,8 +592,8 @@ __global__ void __launch_bounds__(512, 2) k_batched(BTask b, BItems it) {
         const ItemRef r = item_ref(it, item);
         if (r.bin >= BIN_WARP0 && r.bin < BIN_CTA0) {
             bgroup_dispatch(b, r.bin, r.idx, smem, phase);
-        } else if (phase < 2 && r.bin == BIN_DENSE && it.dense_warp) {
-            if constexpr (phase < 2) bdense_warp_item<phase>(b, r.idx, smem);
+        } else if (it.dense_warp && (phase == 2 || r.bin == BIN_DENSE)) {
+            bdense_warp_item<phase>(b, r.bin, r.idx, smem);
         } else {
             const int64_t g = b.cols[b.boff.v[r.bin] + r.idx];
             const int p = find_prob(b.col0s, b.nb, g);
@@ -696,9 +779,21 @@ struct spg_bplan {
 namespace {
 
 // Dense columns of the forward phases are worked one per warp when every
-// product's flags fit kWarpDenseWords words.
+// product's flags fit kWarpDenseWords words.  So are the CTA-level columns of
+// the backward where in addition no column is long enough to hold the launch
+// up on one warp and the warps' flags leave room for two CTAs per SM (a
+// batch step of 12 products of 300 to 4000 rows, forward and backward: 716 us
+// with one 512-thread CTA per column in the backward, 784 us with its walk
+// split into long and short entries, 686 us with one warp per column).
 bool warp_dense(const spg_bplan &P, int phase) {
-    return phase < 2 && P.host.hist[BIN_DENSE] != 0 && P.Wmax <= kWarpDenseWords;
+    if (P.Wmax > kWarpDenseWords) return false;
+    if (phase < 2) return P.host.hist[BIN_DENSE] != 0;
+    bool any = false;
+    for (int b = BIN_CTA0; b < NBINS; ++b) {
+        any |= P.host.hist[b] != 0;
+        if (P.host.maxop[b] > (unsigned long long)kWarpBackwardOps) return false;
+    }
+    return any && (size_t)(P.threads / 32) * al16((size_t)P.Wmax * 8) <= P.smem_optin / 2;
 }
 
 // Items of a phase, heaviest first.
@@ -716,7 +811,9 @@ BItems make_items(const spg_bplan &P, int threads, int phase) {
     it.dense_warp = warp_dense(P, phase) ? 1 : 0;
     add(BIN_DENSE, it.dense_warp ? ceil_div((int64_t)P.host.hist[BIN_DENSE], threads / 32)
                                  : (int64_t)P.host.hist[BIN_DENSE]);
-    for (int c = kNumCtaBins - 1; c >= 0; --c) add(BIN_CTA0 + c, (int64_t)P.host.hist[BIN_CTA0 + c]);
+    for (int c = kNumCtaBins - 1; c >= 0; --c)
+        add(BIN_CTA0 + c, it.dense_warp && phase == 2 ? ceil_div((int64_t)P.host.hist[BIN_CTA0 + c], threads / 32)
+                                                      : (int64_t)P.host.hist[BIN_CTA0 + c]);
     for (int w = kNumWarpBins - 1; w >= 0; --w) {
         const int NG = threads / warp_bin_G(w);
         add(BIN_WARP0 + w, ceil_div((int64_t)P.host.hist[BIN_WARP0 + w], NG));
@@ -763,7 +860,7 @@ size_t phase_smem(const spg_bplan &P, int phase, int threads, int64_t &cap_cta, 
         int64_t mx = (int64_t)P.host.maxnnz[BIN_DENSE];
         for (int c = 0; c < kNumCtaBins; ++c) mx = std::max<int64_t>(mx, (int64_t)P.host.maxnnz[BIN_CTA0 + c]);
         cap_dense = std::min<int64_t>((int64_t)(room / w), mx);
-        if (cta || dense) need = std::max(need, fixed + (size_t)cap_dense * w);
+        if ((cta || dense) && !wd) need = std::max(need, fixed + (size_t)cap_dense * w);
         return need;
     }
     if (dense) need = std::max(need, fixed);

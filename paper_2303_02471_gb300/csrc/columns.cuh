@@ -386,16 +386,30 @@ __device__ __forceinline__ void group_walk_bwd(unsigned mask, const TOps<VT> &o,
     }
 }
 
-// Same chunking and window split as cta_walk (one list of non-empty entries);
-// every lane of a warp calls step(...) once per window from a single call
-// site (p = -1 when idle), so the segmented reduction is warp-wide.
-// pidx: blockDim ints of shared memory.  Contains barriers.
-template <typename VT, typename S>
+// Windows of a long entry a lane of the backward walk gathers at once.
+constexpr int kBwdBatch = 4;
+
+// Backward walk of a CTA over the products of B entries [p0, p1), with
+// cta_walk's chunks, windows and split between long and short entries.
+// lookup(row) gives dC_ij; dA and dB (either may be null) receive the
+// gradients.
+//   * Long entries: a warp takes the entry's windows one after another, every
+//     lane sums a * g over them, and one warp reduction and one add to dB end
+//     the entry's run.  (A segmented reduction per window cost five double
+//     adds and ten shuffles for 32 products: at two FP64 lanes per SM and
+//     clock that was most of the kernel's FP64 time.)
+//   * Short entries share windows: owners are non-decreasing over the lanes
+//     and a segment is shorter than kLongEntry lanes, so a segmented scan of
+//     log2(kLongEntry) steps leaves one add per entry and window.
+// pidx: blockDim ints of shared memory.  Contains barriers: every thread of
+// the CTA must call it.
+template <typename VT, typename L>
 __device__ __forceinline__ void cta_walk_bwd(const TOps<VT> &o, int64_t p0, int64_t p1, const WalkSmem<VT> &w,
-                                             int32_t *pidx, S &&step) {
+                                             int32_t *pidx, VT *dA, VT *dB, L &&lookup) {
     const int T = blockDim.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = T >> 5;
     const unsigned upto = lane == 31 ? 0xffffffffu : ((2u << lane) - 1u);
+    const uint64_t pol = keep_policy();
     for (int64_t base = p0; base < p1; base += T) {
         const int64_t p = base + threadIdx.x;
         int z = 0;
@@ -407,40 +421,102 @@ __device__ __forceinline__ void cta_walk_bwd(const TOps<VT> &o, int64_t p0, int6
             z = (int)(o.Acp[k + 1] - a0);
             bv = o.Bval[p];
         }
-        int v[4] = {z, z > 0 ? 1 : 0, 0, 0};
-        const int mz = z;
+        const bool lng = z >= kLongEntry;
+        // counters: long windows, long entries, short products, short entries
+        int v[4] = {lng ? (z + 31) >> 5 : 0, lng ? 1 : 0, lng ? 0 : z, (!lng && z > 0) ? 1 : 0};
+        const int mine0 = v[0], mine2 = v[2];
         int tot[4];
         cta_incl_scan4(v, w.warp, tot);
+        const int nl = tot[1];
         if (z > 0) {
-            const int i = v[1] - 1;
-            w.key[i] = v[0] - mz;
+            const int i = lng ? v[1] - 1 : nl + v[3] - 1;
+            w.key[i] = lng ? v[0] - mine0 : v[2] - mine2;
+            w.z[i] = z;
             w.a0[i] = a0;
             w.bv[i] = bv;
             pidx[i] = (int32_t)threadIdx.x;
         }
         __syncthreads();
-        const int total = tot[0], nz = tot[1];
-        const int nwin = (total + 31) >> 5;
-        const int win0 = (int)((int64_t)nwin * warp / nw), win1 = (int)((int64_t)nwin * (warp + 1) / nw);
-        if (win0 < win1) {
-            const int qs = win0 << 5;
-            int s = 0, hi = nz - 1;
+        const int WL = tot[0], nsh = tot[3], ZS = tot[2];
+        const int64_t nwin = (int64_t)WL + ((ZS + 31) >> 5);
+        const int win0 = (int)(nwin * warp / nw), win1 = (int)(nwin * (warp + 1) / nw);
+        // ---- long entries: windows [win0, min(win1, WL))
+        const int e1 = win1 < WL ? win1 : WL;
+        if (win0 < e1) {
+            int li = 0, hi = nl - 1;
+            while (li < hi) {
+                const int mid = (li + hi + 1) >> 1;
+                if (w.key[mid] <= win0) li = mid; else hi = mid - 1;
+            }
+            for (int win = win0; win < e1; ++li) {
+                const int e_key = w.key[li], e_z = w.z[li];
+                const int nk = li + 1 < nl ? w.key[li + 1] : 0x7fffffff;
+                const int e_end = nk < e1 ? nk : e1;
+                const int64_t ea = w.a0[li];
+                const VT b = w.bv[li];
+                const int last = (e_end - e_key) << 5;
+                const int i1 = last < e_z ? last : e_z;
+                VT acc = VT(0);
+                for (int idx = ((win - e_key) << 5) + lane; idx - lane < i1; idx += 32 * kBwdBatch) {
+                    int32_t row[kBwdBatch];
+                    VT av[kBwdBatch], g[kBwdBatch];
+#pragma unroll
+                    for (int u = 0; u < kBwdBatch; ++u) {
+                        const int q = idx + 32 * u;
+                        row[u] = q < i1 ? ld_keep(o.Arow + ea + q, pol) : -1;
+                        av[u] = q < i1 && dB ? ld_keep(o.Aval + ea + q, pol) : VT(0);
+                    }
+#pragma unroll
+                    for (int u = 0; u < kBwdBatch; ++u) g[u] = row[u] >= 0 ? lookup(row[u]) : VT(0);
+#pragma unroll
+                    for (int u = 0; u < kBwdBatch; ++u) {
+                        if (row[u] >= 0 && dA) atomicAdd(&dA[ea + idx + 32 * u], b * g[u]);
+                        acc += av[u] * g[u];
+                    }
+                }
+                if (dB) {
+#pragma unroll
+                    for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
+                    if (lane == 0) atomicAdd(&dB[base + pidx[li]], acc);
+                }
+                win = e_end;
+            }
+        }
+        // ---- short entries: windows [max(win0, WL), win1) of the concatenation
+        const int s0w = (win0 > WL ? win0 : WL) - WL, s1w = win1 - WL;
+        if (s0w < s1w) {
+            const int *sk = w.key + nl;
+            const int64_t *sa = w.a0 + nl;
+            const VT *sb = w.bv + nl;
+            const int qs = s0w << 5;
+            int s = 0, hi = nsh - 1;
             while (s < hi) {
                 const int mid = (s + hi + 1) >> 1;
-                if (w.key[mid] <= qs) s = mid; else hi = mid - 1;
+                if (sk[mid] <= qs) s = mid; else hi = mid - 1;
             }
-            for (int win = win0; win < win1; ++win) {
+            for (int win = s0w; win < s1w; ++win) {
                 const int qf = win << 5;
                 const int cand = s + 1 + lane;
-                const int pos = cand < nz ? w.key[cand] - qf : 64;
+                const int pos = cand < nsh ? sk[cand] - qf : 64;
                 const unsigned bits = __reduce_or_sync(0xffffffffu, pos < 32 ? (1u << pos) : 0u);
                 const int own = s + __popc(bits & upto);
                 const int q = qf + lane;
-                const bool on = q < total;
-                const int64_t qa = on ? w.a0[own] + (q - w.key[own]) : 0;
-                const int32_t row = on ? o.Arow[qa] : 0;
-                const VT av = on ? o.Aval[qa] : VT(0);
-                step(row, av, on ? w.bv[own] : VT(0), qa, on ? base + pidx[own] : (int64_t)-1);
+                const bool on = q < ZS;
+                const int64_t qa = on ? sa[own] + (q - sk[own]) : 0;
+                const VT g = on ? lookup(ld_keep(o.Arow + qa, pol)) : VT(0);
+                if (on && dA) atomicAdd(&dA[qa], sb[own] * g);
+                if (dB) {
+                    VT x = on ? ld_keep(o.Aval + qa, pol) * g : VT(0);
+                    const int po = on ? own : -1;
+#pragma unroll
+                    for (int d = 1; d < kLongEntry; d <<= 1) {
+                        const VT xo = __shfl_up_sync(0xffffffffu, x, d);
+                        const int oo = __shfl_up_sync(0xffffffffu, po, d);
+                        if (lane >= d && oo == po) x += xo;
+                    }
+                    const int pn = __shfl_down_sync(0xffffffffu, po, 1);
+                    if (on && (lane == 31 || pn != po)) atomicAdd(&dB[base + pidx[nl + own]], x);
+                }
                 s += __popc(bits) + (__ballot_sync(0xffffffffu, pos == 32) ? 1 : 0);
             }
         }
@@ -493,9 +569,7 @@ __device__ __forceinline__ bool bwd_cta_column(const TOps<VT> &o, int32_t j, int
         const int32_t slot = hash_find(keys, H, row);
         return slot >= 0 ? vals[slot] : VT(0);
     };
-    cta_walk_bwd<VT>(o, o.Bcp[j], o.Bcp[j + 1], w, pidx, [&](int32_t row, VT a, VT b, int64_t qa, int64_t p) {
-        bwd_product<32, VT>(0xffffffffu, row, a, b, qa, p, dA, dB, lookup);
-    });
+    cta_walk_bwd<VT>(o, o.Bcp[j], o.Bcp[j + 1], w, pidx, dA, dB, lookup);
     return ok;
 }
 
@@ -519,15 +593,11 @@ __device__ __forceinline__ void bwd_dense_column(const TOps<VT> &o, int32_t j, i
     __syncthreads();
     if (in_smem) {
         auto lookup = [&](int32_t row) -> VT { return s_dc[bitmap_rank(bm, row)]; };
-        cta_walk_bwd<VT>(o, o.Bcp[j], o.Bcp[j + 1], w, pidx, [&](int32_t row, VT a, VT b, int64_t qa, int64_t p) {
-            bwd_product<32, VT>(0xffffffffu, row, a, b, qa, p, dA, dB, lookup);
-        });
+        cta_walk_bwd<VT>(o, o.Bcp[j], o.Bcp[j + 1], w, pidx, dA, dB, lookup);
     } else {
         const VT *gdc = dC + c0;
         auto lookup = [&](int32_t row) -> VT { return gdc[bitmap_rank(bm, row)]; };
-        cta_walk_bwd<VT>(o, o.Bcp[j], o.Bcp[j + 1], w, pidx, [&](int32_t row, VT a, VT b, int64_t qa, int64_t p) {
-            bwd_product<32, VT>(0xffffffffu, row, a, b, qa, p, dA, dB, lookup);
-        });
+        cta_walk_bwd<VT>(o, o.Bcp[j], o.Bcp[j + 1], w, pidx, dA, dB, lookup);
     }
     for (int64_t e = threadIdx.x; e < nn; e += blockDim.x) bm[Crow[c0 + e] >> 5].x = 0u;
     __syncthreads();

@@ -270,3 +270,44 @@ def test_galerkin_finite_differences_workload5():
             vm[i] -= h
             fd = (loss_of(vp).item() - loss_of(vm).item()) / (2 * h)
             assert abs(fd - grad[i]) <= 1e-6 * max(1.0, abs(grad[i])), (int(i), fd, grad[i])
+
+
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+@pytest.mark.parametrize("heavy", [False, True])
+def test_backward_entry_and_column_lengths(heavy, dtype):
+    """Long and short entries at the edges of their windows and columns of B
+    at the edges of the lanes per entry, alone (one CTA per column) and in a
+    batch (one warp per column; a column of more than 8192 products takes the
+    batch back to one CTA).  The longest sum has 300 terms (u = 6e-8 in
+    float), or 400 for a heavy column's dA: 2.5e-5 bounds its rounding."""
+    import torch
+    from paper_2303_02471_gb300 import ops
+    rng = np.random.default_rng(17)
+    m, lengths = 1037, [0, 1, 15, 16, 17, 31, 32, 33, 127, 128, 129, 300]
+    k = 4 * len(lengths)
+    za = np.array([lengths[i % len(lengths)] for i in range(k)])
+    zb = [0, 1, 2, 3, 4, 5, 8, 9, 16, 17, 31, 32, 33, 40] + ([k] * 3 if heavy else [])
+
+    def matrix(nrows, z):
+        cp = np.concatenate([[0], np.cumsum(z)]).astype(np.int64)
+        rows = np.concatenate([rng.permutation(nrows)[:n] for n in z]).astype(np.int32)
+        return synth.CSC(nrows, len(z), cp, rows, rng.standard_normal(rows.size).astype(dtype))
+    A, B = matrix(m, za), matrix(k, np.array(zb))
+    if heavy:  # one column of B walks every entry of a longer A
+        A = matrix(m, np.maximum(za, 250))
+    tau = 1e-12 if dtype == np.float64 else 2.5e-5
+    dA, dB = upload(A, dtype), upload(B, dtype)
+    C, plan = ops.spgemm(dA, dB, ops.Config(t=1))
+    dc = torch.as_tensor(rng.standard_normal(C.nnz).astype(dtype), device="cuda")
+    got = [ops.spgemm_backward(plan, dA, dB, C, dc)]
+    plan.check()
+    Cs, bplan = ops.spgemm_batched([dA], [dB], ops.Config(t=1))
+    grads = ops.spgemm_batched_backward(bplan, [dA], [dB], Cs, [dc])
+    bplan.check()
+    got.append((grads[0][0], grads[1][0]))
+    Ch, d = C.to_host(), dc.cpu().numpy()
+    want = oracle.backward(A, B, Ch, d)
+    scale = oracle.backward(A.with_values(np.abs(A.values)), B.with_values(np.abs(B.values)), Ch, np.abs(d))
+    for pair in got:
+        for g, r, s in zip(pair, want, scale):
+            assert np.all(np.abs(g.cpu().numpy().astype(np.float64) - r) <= tau * s)
