@@ -311,3 +311,28 @@ def test_backward_entry_and_column_lengths(heavy, dtype):
     for pair in got:
         for g, r, s in zip(pair, want, scale):
             assert np.all(np.abs(g.cpu().numpy().astype(np.float64) - r) <= tau * s)
+
+
+@pytest.mark.parametrize("lengths", [[0, 1, 2], [1, 3, 4, 2], [5, 7, 8, 1], [9, 2, 31, 32, 33, 64, 65, 8],
+                                     [255, 256, 257, 1, 0, 512, 513]])
+def test_transpose_row_lengths(lengths):
+    """Rows at the edges of the sorts (a lane's, a warp's, a CTA's), mixed
+    within one warp, with unsorted columns."""
+    from paper_2303_02471_gb300 import ops
+    rng = np.random.default_rng(11)
+    m, n = 137, 600
+    D = np.zeros((m, n))
+    for i in range(m):
+        D[i, rng.permutation(n)[:lengths[i % len(lengths)]]] = 1.0
+    cols, rows = np.nonzero(D.T)
+    M = synth.from_coo(m, n, rows, cols, rng.standard_normal(rows.size))
+    for j in range(n):  # any order inside a column
+        lo, hi = M.colptr[j], M.colptr[j + 1]
+        M.rowidx[lo:hi] = M.rowidx[lo:hi][::-1].copy()
+    T, perm = ops.csc_transpose(upload(M))
+    R, q = oracle.transpose(M)
+    Th = T.to_host()
+    assert np.array_equal(Th.colptr, R.colptr)
+    assert np.array_equal(Th.rowidx, R.rowidx)
+    assert np.array_equal(Th.values, R.values)
+    assert np.array_equal(perm.cpu().numpy(), q)
