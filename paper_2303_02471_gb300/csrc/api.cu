@@ -39,7 +39,7 @@ size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 
 struct Layout {
     size_t ctrl = 0, op = 0, cols = 0, tiles = 0, scratch = 0, cache = 0, total = 0;
-    size_t rmark = 0, rtiles = 0, rmap = 0, rinv = 0, arow = 0;
+    size_t rmark = 0, rmark_end = 0, zlen = 0, rtiles = 0, rmap = 0, rinv = 0, arow = 0;
     size_t scratch_stride = 0;
     int64_t scratch_ctas = 0;
     int64_t cache_cols = 0;
@@ -53,36 +53,27 @@ spg_config normalized(const spg_config *cfg) {
     return c;
 }
 
-// Default threshold: the dense SPA pays O(m / 32) words per column (flag
-// bitmap prefix and sorted extraction), so a column goes dense once its
-// product count reaches m / 512 (the crossover measured on GB300), within
-// [257, hash_cta_max + 1]; m counts the rows the forward passes number.
-int64_t effective_t(const spg_config &c, int64_t m) {
-    if (c.t >= 0) return c.t;
-    int64_t t = (m + 511) / 512;
-    if (t > (int64_t)c.hash_cta_max + 1) t = (int64_t)c.hash_cta_max + 1;
-    if (t < 257) t = 257;
-    return t;
-}
-
 bool valid_hash_max(int32_t h) {
     return h == 256 || h == 512 || h == 1024 || h == 2048 || h == 4096 || h == 8192;
 }
 
-Layout make_layout(int64_t m, int64_t nB, int64_t nnzA, int dtype, const spg_config &c, int sms) {
+Layout make_layout(int64_t m, int64_t nA, int64_t nB, int64_t nnzA, int dtype, const spg_config &c, int sms) {
     Layout L;
     const size_t w = dtype == SPG_F64 ? 8 : 4;
     const int64_t W = ceil_div(m, 32);
     const int64_t hmax = c.hash_cta_max;
     size_t off = 0;
     L.ctrl = off; off = align256(off + sizeof(Ctrl));
+    // row compaction: a mark per row with entries (cleared together with the
+    // control block), counts per tile of rows, the map to compact rows and
+    // back, and A's rows renumbered; the lengths of A's columns
+    L.rmark = off; off = align256(off + row_mark_bytes(m));
+    L.rmark_end = off;
+    L.zlen = off; off = align256(off + (size_t)nA * 4);
     L.op = off; off = align256(off + (size_t)nB * 8);
     L.cols = off; off = align256(off + (size_t)nB * 4);
     L.tiles = off; off = align256(off + (size_t)scan_tile_count(nB) * 8);
-    // row compaction: marks (scanned in place), the map to compact rows and
-    // back, and A's rows renumbered
-    L.rmark = off; off = align256(off + (size_t)m * 8);
-    L.rtiles = off; off = align256(off + (size_t)scan_tile_count(m) * 8);
+    L.rtiles = off; off = align256(off + (size_t)row_tile_count(m) * 4);
     L.rmap = off; off = align256(off + (size_t)m * 4);
     L.rinv = off; off = align256(off + (size_t)m * 4);
     L.arow = off; off = align256(off + (size_t)nnzA * 4);
@@ -91,7 +82,7 @@ Layout make_layout(int64_t m, int64_t nB, int64_t nnzA, int dtype, const spg_con
     const int64_t reach = std::min<int64_t>(std::max<int64_t>(nnzA, 1), std::max<int64_t>(m, 1));
     // hash table keys + values + word list of the extraction (numeric)
     size_t tab = (size_t)num_slots(std::min<int64_t>(hmax, reach), c.table_slots_pct) * (8 + w) + 64;
-    if (effective_t(c, m) > hmax + 1) {
+    if (effective_t(c.t, hmax, m) > hmax + 1) {
         const size_t sym = (size_t)global_sym_slots(reach, m) * 4;
         const size_t num = (size_t)num_slots(reach, c.table_slots_pct) * (8 + w) + 64;
         tab = std::max(tab, std::max(sym, num));
@@ -183,6 +174,22 @@ struct spg_plan {
                      cudaStream_t s) {
         return handle_readback(h, dst0, src0, n0, dst1, src1, n1, s);
     }
+    // C's column pointers from the columns' counts, with nnz(C) and the
+    // control block read back (from the scan's last kernel).
+    cudaError_t scan_and_read(int64_t *C_colptr, cudaStream_t s) {
+        if (nB <= 0) return read(&nnzC, C_colptr, sizeof(int64_t), &host, ctrl(), sizeof(Ctrl), s);
+        struct {
+            int64_t last;
+            Ctrl ctrl;
+        } got;
+        const cudaError_t e = handle_mirrored(h, &got, sizeof(got), s, [&](unsigned char *host_mem) {
+            return launch_inclusive_scan(C_colptr + 1, nB, tiles(), s, ctrl(), host_mem);
+        });
+        if (e != cudaSuccess) return e;
+        nnzC = got.last;
+        host = got.ctrl;
+        return cudaSuccess;
+    }
     int64_t nonempty_bins() const {
         int64_t n = 0;
         for (int b = 1; b < NBINS; ++b) n += host.hist[b] ? 1 : 0;
@@ -195,6 +202,7 @@ struct spg_plan {
     int64_t *tiles() const { return reinterpret_cast<int64_t *>(ws + L.tiles); }
     unsigned char *scratch() const { return ws + L.scratch; }
     int64_t *rmark() const { return reinterpret_cast<int64_t *>(ws + L.rmark); }
+    uint32_t *zlen() const { return reinterpret_cast<uint32_t *>(ws + L.zlen); }
     int32_t *rmap() const { return reinterpret_cast<int32_t *>(ws + L.rmap); }
     int32_t *rinv() const { return reinterpret_cast<int32_t *>(ws + L.rinv); }
     int32_t *arow() const { return reinterpret_cast<int32_t *>(ws + L.arow); }
@@ -304,7 +312,7 @@ spg_status spgemm_workspace_size(const spg_csc *A, const spg_csc *B, const spg_c
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return SPG_ERR_CUDA;
     DeviceInfo di = device_info(dev);
-    *bytes = make_layout(A->nrows, B->ncols, A->nnz, A->dtype, c, di.sms).total;
+    *bytes = make_layout(A->nrows, A->ncols, B->ncols, A->nnz, A->dtype, c, di.sms).total;
     return SPG_OK;
 }
 
@@ -368,7 +376,7 @@ static spg_status prepare(spg_handle *handle, const spg_csc *A, const spg_csc *B
     P->nnzA = A->nnz; P->nnzB = B->nnz;
     P->dtype = A->dtype;
     P->cfg = c;
-    P->L = make_layout(P->mA, P->nB, P->nnzA, P->dtype, c, P->dev.sms);
+    P->L = make_layout(P->mA, P->nA, P->nB, P->nnzA, P->dtype, c, P->dev.sms);
     if (ws_bytes < P->L.total) { delete P; return SPG_ERR_WORKSPACE; }
     P->ws = static_cast<unsigned char *>(workspace);
     P->ws_bytes = ws_bytes;
@@ -382,55 +390,32 @@ static spg_status prepare(spg_handle *handle, const spg_csc *A, const spg_csc *B
         if (e_ != cudaSuccess) { delete P; return SPG_ERR_CUDA; }     \
     } while (0)
 
-    CK(cudaMemsetAsync(ctrl, 0, sizeof(Ctrl), s));
-    if (c.validate) {
-        const int vg = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(std::max(A->nnz, A->ncols + 1), 256), 8 * P->dev.sms));
-        k_validate<<<vg, 256, 0, s>>>(A->colptr, A->rowidx, A->nrows, A->ncols, A->nnz, 0, ctrl);
-        const int vb = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(std::max(B->nnz, B->ncols + 1), 256), 8 * P->dev.sms));
-        k_validate<<<vb, 256, 0, s>>>(B->colptr, B->rowidx, B->nrows, B->ncols, B->nnz, 1, ctrl);
-        CK(cudaGetLastError());
-    }
-    // Row compaction of the forward passes (bounds-checked, so it may run
-    // before the validation outcome): a row of A without entries has none in
-    // C, and the dense flags, their cache and the CTA bitmaps then span only
-    // the rows that hold entries.
-    int64_t mC = P->mA;
-    const bool try_compact = P->mA > 0 && P->nnzA > 0;
-    if (try_compact) {
-        CK(cudaMemsetAsync(P->rmark(), 0, (size_t)P->mA * 8, s));
-        const int ga = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(A->nnz, 256), 8 * P->dev.sms));
-        k_row_mark<<<ga, 256, 0, s>>>(A->rowidx, A->nnz, P->mA, P->rmark());
-        CK(cudaGetLastError());
-        CK(launch_inclusive_scan(P->rmark(), P->mA, reinterpret_cast<int64_t *>(P->ws + P->L.rtiles), s));
-    }
-    // one read: the validation outcome (a malformed colptr would make the
-    // walks read out of bounds: stop here) and the count of rows with entries
-    CK(P->read(&P->host, ctrl, sizeof(Ctrl), try_compact ? &mC : nullptr,
-               try_compact ? P->rmark() + (P->mA - 1) : nullptr, try_compact ? sizeof(int64_t) : 0, s));
+    // One chain without the host in it: A checked and its rows marked, the
+    // rows numbered, A renumbered where compaction applies (a row of A without
+    // entries has none in C, so the dense flags, their cache and the CTA
+    // bitmaps span only the rows that hold entries) with Op_j and the bins
+    // counted and B checked, the column lists.  Each kernel leaves alone what
+    // an earlier one found malformed; the host reads the outcome once.
+    CK(cudaMemsetAsync(ctrl, 0, P->L.rmark_end - P->L.ctrl, s));
+    int launches = 0;
+    const int ga = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(std::max(A->nnz, A->ncols + 1), 1024), 8 * P->dev.sms));
+    k_check_rows<<<ga, 256, 0, s>>>(A->colptr, A->rowidx, A->nrows, A->ncols, A->nnz, c.validate, P->rmark(), P->zlen(),
+                                     ctrl);
+    CK(cudaGetLastError());
+    if (P->mA > 0 && P->nnzA > 0)
+        CK(launch_row_index(P->rmark(), P->mA, reinterpret_cast<int32_t *>(P->ws + P->L.rtiles), P->rmap(), P->rinv(),
+                            ctrl, &launches, s));
+    const CountArgs args{B->colptr, B->rowidx, P->zlen(), A->rowidx, P->mA, P->nA, P->nB, P->nnzA, P->nnzB,
+                         P->rmap(), P->arow(), c.t, hmax, c.group_promote, c.validate, P->op(), C_colptr};
+    CK(launch_count_bin(args, P->dev.sms, ctrl, s));
+    CK(handle_mirrored(P->h, &P->host, sizeof(Ctrl), s, [&](unsigned char *host) {
+        return launch_bin_scatter(args, scatter ? P->cols() : nullptr, ctrl, host, s);
+    }));
     if (P->host.err) { st = (spg_status)P->host.err; delete P; return st; }
-    P->compact = try_compact && mC > 0 && mC * 10 <= P->mA * 9;
-    P->mC = P->compact ? mC : P->mA;
-    if (P->compact) {
-        // the map to compact rows and back, and A's rows renumbered (rows
-        // out of range were rejected by the validation, or are reported here)
-        const int ga = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(A->nnz, 256), 8 * P->dev.sms));
-        const int gm = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(P->mA, 256), 8 * P->dev.sms));
-        k_row_map<<<gm, 256, 0, s>>>(P->rmark(), P->mA, P->rmap(), P->rinv());
-        k_row_remap<<<ga, 256, 0, s>>>(A->rowidx, A->nnz, P->rmap(), P->mA, P->arow(), ctrl);
-        CK(cudaGetLastError());
-    }
-    P->t_eff = effective_t(c, P->mC);
-    if (P->nB > 0) {
-        // a warp per 32 columns, 8 warps per CTA
-        const int g = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(P->nB, 256), 16 * (int64_t)P->dev.sms));
-        k_count_bin<<<g, 256, 0, s>>>(B->colptr, B->rowidx, A->colptr, P->nB, P->t_eff, hmax, c.group_promote, P->mC,
-                                      column_deal_mult(P->nB), P->op(), C_colptr, ctrl);
-        CK(cudaGetLastError());
-    } else {
-        CK(cudaMemsetAsync(C_colptr, 0, sizeof(int64_t), s));
-    }
-    CK(P->read(&P->host, ctrl, sizeof(Ctrl), nullptr, nullptr, 0, s));
-    if (P->host.err) { st = (spg_status)P->host.err; delete P; return st; }
+    const RowRule rows = row_rule((int64_t)P->host.mrows, P->mA);
+    P->compact = rows.compact;
+    P->mC = rows.m;
+    P->t_eff = effective_t(c.t, hmax, P->mC);
     // the walks index a column's products with 32-bit offsets
     for (int b = 0; b < NBINS; ++b)
         if (P->host.maxop[b] >= (1ULL << 31)) { delete P; return SPG_ERR_UNSUPPORTED; }
@@ -441,22 +426,15 @@ static spg_status prepare(spg_handle *handle, const spg_csc *A, const spg_csc *B
         const int64_t n = b == BIN_EMPTY ? 0 : (int64_t)P->host.hist[b];
         P->off.v[b + 1] = P->off.v[b] + n;
     }
-    if (scatter && P->nB > 0) {
-        k_bin_scatter<<<(unsigned)ceil_div(P->nB, 256), 256, 0, s>>>(P->op(), P->nB, P->t_eff, hmax, c.group_promote,
-                                                                     P->off, P->cols(), ctrl);
-        CK(cudaGetLastError());
-    }
-    CK(cudaMemsetAsync(&ctrl->work, 0, sizeof(ctrl->work), s));
 #undef CK
     // the numeric phase (and the single pass) take ESC unless hash tables
     // were asked for; the symbolic phase counts with ESC when asked, and by
     // default in the bins that ESC sorts by rank (sym_bin)
     if (c.small_accumulator != SPG_ACC_HASH)
         for (int b = BIN_WARP0; b < BIN_CTA0; ++b) P->esc[b] = esc_shape(b, P->mC, P->esc_shape_of[b]);
-    // validation, row marks (mark, 3 scan kernels) and, when compacting,
-    // map and remap, the two control reads, Op counting + scatter
-    P->sym_launches = (c.validate ? 2 : 0) + (try_compact ? 4 : 0) + (P->compact ? 2 : 0) + 2 +
-                      (P->nB > 0 ? 1 + (scatter ? 1 : 0) : 0);
+    // A's checks and row marks, the row index, Op counting, the scatter with
+    // the control read
+    P->sym_launches = 3 + launches;
     *out = P;
     return SPG_OK;
 }
@@ -527,8 +505,7 @@ spg_status spgemm_symbolic(spg_handle *handle, const spg_csc *A, const spg_csc *
         }
         CK(first);
     }
-    CK(launch_inclusive_scan(C_colptr + 1, P->nB, P->tiles(), s));
-    CK(P->read(&P->nnzC, C_colptr + P->nB, sizeof(int64_t), &P->host, ctrl, sizeof(Ctrl), s));
+    CK(P->scan_and_read(C_colptr, s));
 #undef CK
     if (P->host.err) { st = (spg_status)P->host.err; delete P; return st; }
     for (int b = 1; b < NBINS; ++b) {
@@ -538,8 +515,8 @@ spg_status spgemm_symbolic(spg_handle *handle, const spg_csc *A, const spg_csc *
                                          P->L.scratch_ctas);
     }
     P->num_geo_ready = true;
-    // the preparation, 3 scan kernels, the control read, the bins
-    P->sym_launches += 4 + P->nonempty_bins();
+    // the preparation, the scan with the control read, the bins
+    P->sym_launches += std::max(1, scan_launches(P->nB)) + P->nonempty_bins();
     *nnzC = P->nnzC;
     *plan_out = P;
     return SPG_OK;
@@ -689,13 +666,13 @@ spg_status spgemm_single_pass(spg_handle *handle, const spg_csc *A, const spg_cs
                P->compact ? P->rinv() : nullptr};
     st = run_numeric(P, o, soff, C_colptr, reinterpret_cast<int32_t *>(P->ws + P->srow_at), P->ws + P->sval_at, s);
     if (st != SPG_OK) { delete P; return st; }
-    CK(launch_inclusive_scan(C_colptr + 1, P->nB, P->tiles(), s));
-    CK(P->read(&P->nnzC, C_colptr + P->nB, sizeof(int64_t), &P->host, ctrl, sizeof(Ctrl), s));
+    CK(P->scan_and_read(C_colptr, s));
 #undef CK
     if (P->host.err) { st = (spg_status)P->host.err; delete P; return st; }
-    // the preparation, slot caps and 3 scan kernels, the bins, 3 scan
-    // kernels and the control read
-    P->sym_launches += (P->nB > 0 ? 4 : 0) + P->nonempty_bins() + 4;
+    // the preparation, slot caps and their scan, the bins, the scan with the
+    // control read
+    P->sym_launches += (P->nB > 0 ? 1 + scan_launches(P->nB) : 0) + P->nonempty_bins() +
+                       std::max(1, scan_launches(P->nB));
     *nnzC = P->nnzC;
     *plan_out = P;
     return SPG_OK;

@@ -3,6 +3,7 @@
 // mapped pinned buffer of the small synchronising reads.  Host code only.
 #pragma once
 
+#include <cstring>
 #include <mutex>
 
 #include "kernels.cuh"
@@ -60,6 +61,23 @@ inline cudaError_t handle_readback(spg_handle *h, void *dst0, const void *src0, 
     if (!h) return readback(nullptr, dst0, src0, n0, dst1, src1, n1, s);
     std::lock_guard<std::mutex> lock(h->mu);
     return readback(&h->mirror, dst0, src0, n0, dst1, src1, n1, s);
+}
+
+// A read that the caller's last kernel makes itself: launch(dev) enqueues it
+// with the mapped mirror's device address, the stream is synchronised, and
+// `n` bytes go to dst (one launch fewer than handle_readback).
+template <typename F>
+inline cudaError_t handle_mirrored(spg_handle *h, void *dst, size_t n, cudaStream_t s, F &&launch) {
+    std::unique_lock<std::mutex> lock;
+    if (h) lock = std::unique_lock<std::mutex>(h->mu);
+    Mirror *m = h ? &h->mirror : thread_mirror();
+    if (!m) return cudaErrorInvalidDevice;
+    cudaError_t e;
+    if ((e = m->reserve(n)) != cudaSuccess) return e;
+    if ((e = launch(static_cast<unsigned char *>(m->dev))) != cudaSuccess) return e;
+    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
+    std::memcpy(dst, m->host, n);
+    return cudaSuccess;
 }
 
 }  // namespace spg

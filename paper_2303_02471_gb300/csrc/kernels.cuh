@@ -773,15 +773,45 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity, long l
 
 // ------------------------------------------------------------ launchers
 // Row compaction.  Rows of A without entries have none in C = A B, so the
-// forward passes may number only the rows that hold entries: mark[r] = 1 for
-// every row of an entry (in range), an inclusive scan of mark gives the count,
-// k_row_map writes map[r] (compact index or -1) and inv[compact] = r, and
-// k_row_remap rewrites A's rows through map, reporting a row without a
-// compact index (kDetailRowMap).
-__global__ void k_row_mark(const int32_t *Arow, int64_t nnz, int64_t m, int64_t *mark);
-__global__ void k_row_map(const int64_t *incl, int64_t m, int32_t *map, int32_t *inv);
+// forward passes may number only the rows that hold entries: k_check_rows sets
+// a mark per row of an entry (and checks A and writes its columns' lengths),
+// launch_row_index counts them (ctrl->mrows) and, where compaction applies,
+// writes map[r] (compact index or -1) and inv[compact] = r; k_row_remap
+// rewrites A's rows through map, reporting a row without a compact index
+// (kDetailRowMap).  mark: row_mark_bytes(m) zeroed bytes, 16-byte aligned;
+// counts: row_tile_count(m) ints.
+__global__ void k_check_rows(const int64_t *cp, const int32_t *row, int64_t nrows, int64_t ncols, int64_t nnz,
+                             int validate, int64_t *mark, uint32_t *zlen, Ctrl *ctrl);
+size_t row_mark_bytes(int64_t m);
+int64_t row_tile_count(int64_t m);
+cudaError_t launch_row_index(const int64_t *mark, int64_t m, int32_t *counts, int32_t *map, int32_t *inv,
+                             Ctrl *ctrl, int *launches, cudaStream_t s);
 __global__ void k_row_remap(const int32_t *Arow, int64_t nnz, const int32_t *map, int64_t m, int32_t *out,
                             Ctrl *ctrl);
+
+// The rows the forward passes number, from the count of rows with entries:
+// compact where that saves at least a tenth of them.  The same on the device
+// (which goes on without the host) and on the host.
+struct RowRule {
+    int64_t m;
+    bool compact;
+};
+__host__ __device__ inline RowRule row_rule(int64_t with_entries, int64_t m) {
+    const bool c = with_entries > 0 && with_entries * 10 <= m * 9;
+    return RowRule{c ? with_entries : m, c};
+}
+
+// Threshold of a product (t < 0: the default).  The dense SPA pays O(m / 32)
+// words per column (flag bitmap prefix and sorted extraction), so a column
+// goes dense once its product count reaches m / 512 (the crossover measured
+// on GB300), within [257, hash_cta_max + 1]; m counts the rows the forward
+// passes number.
+__host__ __device__ inline int64_t effective_t(int64_t t, int64_t hmax, int64_t m) {
+    if (t >= 0) return t;
+    t = (m + 511) / 512;
+    if (t > hmax + 1) t = hmax + 1;
+    return t < 257 ? 257 : t;
+}
 
 // Mapped pinned host buffer of small device -> host reads, grown on demand
 // (at least 64 KiB).
@@ -793,6 +823,9 @@ struct Mirror {
     cudaError_t reserve(size_t need);
 };
 
+// The calling host thread's mirror for the current device (nullptr: none).
+Mirror *thread_mirror();
+
 // Small device -> host reads (control blocks, counts): a one-CTA kernel
 // copies src0[0..n0) and src1[0..n1) into the mapped pinned mirror `m` (NULL:
 // one of the calling host thread for the current device), the stream is
@@ -801,16 +834,37 @@ struct Mirror {
 // has in flight on other streams.
 cudaError_t readback(Mirror *m, void *dst0, const void *src0, size_t n0, void *dst1, const void *src1, size_t n1,
                      cudaStream_t s);
-cudaError_t launch_inclusive_scan(int64_t *x, int64_t n, int64_t *tile_sums, cudaStream_t s);
+// Inclusive scan of x[0..n) in place (tile_sums: scan_tile_count(n) values).
+// With `host` (mapped host memory) the last launch also writes x[n - 1] and
+// then the control block there.
+cudaError_t launch_inclusive_scan(int64_t *x, int64_t n, int64_t *tile_sums, cudaStream_t s,
+                                  const Ctrl *ctrl = nullptr, unsigned char *host = nullptr);
 int64_t scan_tile_count(int64_t n);
+int scan_launches(int64_t n);
 
-__global__ void k_validate(const int64_t *cp, const int32_t *row, int64_t nrows, int64_t ncols,
-                           int64_t nnz, int which, Ctrl *ctrl);
-__global__ void k_count_bin(const int64_t *Bcp, const int32_t *Brow, const int64_t *Acp, int64_t nB,
-                            int64_t t, int64_t hmax, int promote, int64_t mrows, int64_t mult, int64_t *op,
-                            int64_t *Ccp, Ctrl *ctrl);
+// Op counting, binning and B's checks (prep.cu).
+struct CountArgs {
+    const int64_t *Bcp;
+    const int32_t *Brow;
+    const uint32_t *zlen;  // lengths of A's columns
+    const int32_t *Arow;
+    int64_t mA, nA, nB, nnzA, nnzB;
+    const int32_t *rmap;  // row compaction: the map and A's renumbered rows
+    int32_t *arow;
+    int64_t t, hmax;      // the configuration's threshold (< 0: default) and hash_cta_max
+    int promote, validate;
+    int64_t *op, *Ccp;
+    // set by the launcher: the deal of the columns, columns per warp
+    int64_t mult = 1;
+    unsigned long long inv = 0;
+    int cols = 32;
+};
+cudaError_t launch_count_bin(const CountArgs &a, int sms, Ctrl *ctrl, cudaStream_t s);
+// bin_cols null: only the control block goes to the host's mirror.
+cudaError_t launch_bin_scatter(const CountArgs &a, int32_t *bin_cols, Ctrl *ctrl, unsigned char *host,
+                               cudaStream_t s);
 // Multiplier coprime to n (n >= 1) near n times the golden ratio's fraction,
-// dealing the columns of k_count_bin over the warps.
+// dealing k_count_bin's runs of columns over the CTAs.
 int64_t column_deal_mult(int64_t n);
 __global__ void k_slot_caps(const int64_t *op, int64_t nB, int64_t mrows, int64_t *caps);
 // Single pass: C's entries from the slots (two launches: the first column
@@ -820,9 +874,6 @@ cudaError_t launch_slot_copy(int64_t nB, int64_t nnzC, const int64_t *Ccp, const
                              const int32_t *srow, const void *sval, int32_t *Crow, void *Cval, int w, int sms,
                              cudaStream_t s);
 int64_t copy_tile_count(int64_t n);
-__global__ void k_bin_scatter(const int64_t *op, int64_t nB, int64_t t, int64_t hmax, int promote,
-                              BinOffsets off, int32_t *bin_cols, Ctrl *ctrl);
-
 // Geometry of one phase (symbolic / numeric / backward) of one bin.
 struct Geo {
     int threads = 0;       // threads per CTA

@@ -1,5 +1,5 @@
 // Preprocessing kernels of the column-wise SpGEMM (arXiv 2303.02471):
-// input validation, the operation count Op_j with binning (Section 3.1's
+// input validation, row compaction, the operation count Op_j with binning (Section 3.1's
 // "Sorting" pre-pass, done as a bucket pass), per-bin column lists, and the
 // int64 scan that turns per-column counts into C's column pointers.
 #include <cstring>
@@ -8,48 +8,211 @@
 
 namespace spg {
 
-// CSC well-formedness (Section 2.1): colptr[0] = 0, colptr[n] = nnz,
-// colptr non-decreasing, rows in [0, nrows).
-__global__ void k_validate(const int64_t *__restrict__ cp, const int32_t *__restrict__ row,
-                           int64_t nrows, int64_t ncols, int64_t nnz, int which, Ctrl *ctrl) {
+// CSC well-formedness of A (Section 2.1: colptr[0] = 0, colptr[n] = nnz,
+// colptr non-decreasing, rows in [0, nrows)), its columns' lengths as 32-bit
+// integers for the Op count's gathers, and a mark per row that holds an entry,
+// in one pass over A.  A mark is a plain store of eight bytes: stores to one
+// L2 sector from many SMs take turns, so narrow marks lose (bytes took 133 us
+// for the 4.7M entries of the very sparse product and 370 us for the skewed
+// rows of R-MAT 2^18, bits set by atomics 46 and 25 us, so 30 and 42 us).
+constexpr int kCheckUnroll = 4;
+
+__global__ void __launch_bounds__(256) k_check_rows(const int64_t *__restrict__ cp, const int32_t *__restrict__ row,
+                                                   int64_t nrows, int64_t ncols, int64_t nnz, int validate,
+                                                   int64_t *__restrict__ mark, uint32_t *__restrict__ zlen,
+                                                   Ctrl *ctrl) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     for (int64_t j = tid; j <= ncols; j += stride) {
-        int64_t c = cp[j];
-        if ((j == 0 && c != 0) || (j == ncols && c != nnz) || (j < ncols && cp[j + 1] < c) || c < 0)
-            set_error(ctrl, SPG_ERR_INVALID, which * 2 + 0, j);
+        const int64_t c = cp[j], c1 = j < ncols ? cp[j + 1] : c;
+        if (j < ncols) zlen[j] = (uint32_t)(c1 - c);
+        if (validate && ((j == 0 && c != 0) || (j == ncols && c != nnz) || c1 < c || c < 0))
+            set_error(ctrl, SPG_ERR_INVALID, 0, j);
     }
-    for (int64_t e = tid; e < nnz; e += stride) {
-        int32_t r = row[e];
-        if (r < 0 || (int64_t)r >= nrows) set_error(ctrl, SPG_ERR_INVALID, which * 2 + 1, e);
+    for (int64_t e0 = tid; e0 < nnz; e0 += kCheckUnroll * stride) {
+        int32_t r[kCheckUnroll];
+#pragma unroll
+        for (int u = 0; u < kCheckUnroll; ++u) r[u] = e0 + u * stride < nnz ? row[e0 + u * stride] : 0;
+#pragma unroll
+        for (int u = 0; u < kCheckUnroll; ++u) {
+            if (e0 + u * stride >= nnz) continue;
+            if (r[u] >= 0 && (int64_t)r[u] < nrows) mark[r[u]] = 1;
+            else if (validate) set_error(ctrl, SPG_ERR_INVALID, 1, e0 + u * stride);
+        }
     }
 }
 
-// Op_j = sum over stored B_kj of Z^A_k (Section 3.1), its bin, the bin
-// histogram and the total product count.  Empty columns get nnz 0 here.
-//
-// A warp takes 32 columns, one per lane.  The columns are dealt through a
-// permutation (index times `mult` modulo nB, mult coprime to nB) so that the
-// heavy columns of a skewed matrix, which sit together (or, in R-MAT, at
-// indices with few one bits), spread over the warps.  Columns with more than
-// 32 B entries are walked by the whole warp one after another, its loads
-// strided over the lanes; the others' entries are walked 32 at a time as one
-// flattened sequence (the owner of an entry is found by a search over the
-// lanes' entry offsets) and the Z^A_k of an owner's lanes are summed by a
-// segmented warp scan.  Per-bin statistics are summed over the warp before
-// one shared atomic per bin present.
-constexpr int kCountLong = 32;
+// Rows with entries numbered in ascending order, where compaction applies
+// (row_rule): map[r] = compact row or -1, inv[compact] = r.  ctrl->mrows =
+// their count.  A CTA takes a tile of kRowTile rows; the rows of the other
+// tiles are counted from the marks themselves up to kRowRecount tiles (which
+// saves a launch), else from the tiles' counts.  The marks are padded with
+// zeros to whole tiles.
+constexpr int kRowTile = 2048;
+constexpr int kRowThreads = 256;
+constexpr int kRowRecount = 8;
+constexpr int kRowPer = kRowTile / kRowThreads;  // consecutive rows of a thread
 
-__global__ void k_count_bin(const int64_t *__restrict__ Bcp, const int32_t *__restrict__ Brow,
-                            const int64_t *__restrict__ Acp, int64_t nB, int64_t t, int64_t hmax, int promote,
-                            int64_t mrows,
-                            int64_t mult, int64_t *__restrict__ op, int64_t *__restrict__ Ccp, Ctrl *ctrl) {
+// The marks of thread threadIdx.x in tile `tile`, as bits.
+__device__ __forceinline__ uint32_t row_bits(const ulonglong2 *__restrict__ marks, int64_t tile) {
+    uint32_t b = 0;
+#pragma unroll
+    for (int i = 0; i < kRowPer / 2; ++i) {
+        const ulonglong2 v = marks[(tile * kRowThreads + threadIdx.x) * (kRowPer / 2) + i];
+        b |= ((uint32_t)v.x | ((uint32_t)v.y << 1)) << (2 * i);
+    }
+    return b;
+}
+
+__global__ void __launch_bounds__(kRowThreads) k_row_counts(const ulonglong2 *__restrict__ marks,
+                                                           int32_t *__restrict__ counts) {
+    __shared__ int s_n;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    const int w = __reduce_add_sync(0xffffffffu, __popc(row_bits(marks, blockIdx.x)));
+    if ((threadIdx.x & 31) == 0) atomicAdd(&s_n, w);
+    __syncthreads();
+    if (threadIdx.x == 0) counts[blockIdx.x] = s_n;
+}
+
+__global__ void __launch_bounds__(kRowThreads) k_row_index(const ulonglong2 *__restrict__ marks, int64_t m,
+                                                          const int32_t *__restrict__ counts,
+                                                          int32_t *__restrict__ map, int32_t *__restrict__ inv,
+                                                          Ctrl *ctrl) {
+    __shared__ int s_warp[kRowThreads / 32];
+    __shared__ int s_before, s_all;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) s_before = s_all = 0;
+    __syncthreads();
+    // rows with entries before the tile, and of all tiles
+    int before = 0, all = 0;
+    if (counts) {
+        for (int64_t i = threadIdx.x; i < gridDim.x; i += kRowThreads) {
+            const int n = counts[i];
+            all += n;
+            if (i < blockIdx.x) before += n;
+        }
+    } else {
+        for (int64_t t = 0; t < gridDim.x; ++t) {
+            const int n = __popc(row_bits(marks, t));
+            all += n;
+            if (t < blockIdx.x) before += n;
+        }
+    }
+    before = __reduce_add_sync(0xffffffffu, before);
+    all = __reduce_add_sync(0xffffffffu, all);
+    if (lane == 0) {
+        atomicAdd(&s_before, before);
+        atomicAdd(&s_all, all);
+    }
+    const uint32_t bits = row_bits(marks, blockIdx.x);
+    const int c = __popc(bits);
+    int incl = c;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int o = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += o;
+    }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->mrows = (unsigned long long)s_all;
+    if (!row_rule(s_all, m).compact) return;
+    int at = s_before + incl - c;
+    for (int i = 0; i < warp; ++i) at += s_warp[i];
+    const int64_t r0 = (int64_t)blockIdx.x * kRowTile + kRowPer * threadIdx.x;
+#pragma unroll
+    for (int i = 0; i < kRowPer; ++i) {
+        if (r0 + i >= m) break;
+        const bool in = (bits >> i) & 1u;
+        map[r0 + i] = in ? at : -1;
+        if (in) inv[at++] = (int32_t)(r0 + i);
+    }
+}
+
+size_t row_mark_bytes(int64_t m) { return (size_t)ceil_div(m, kRowTile) * kRowTile * sizeof(int64_t); }
+int64_t row_tile_count(int64_t m) { return ceil_div(m, kRowTile) + 1; }
+
+cudaError_t launch_row_index(const int64_t *mark, int64_t m, int32_t *counts, int32_t *map, int32_t *inv,
+                             Ctrl *ctrl, int *launches, cudaStream_t s) {
+    const int64_t tiles = ceil_div(m, kRowTile);
+    if (tiles <= 0) return cudaSuccess;
+    const ulonglong2 *marks = reinterpret_cast<const ulonglong2 *>(mark);
+    const bool direct = tiles <= kRowRecount;
+    if (!direct) k_row_counts<<<(unsigned)tiles, kRowThreads, 0, s>>>(marks, counts);
+    k_row_index<<<(unsigned)tiles, kRowThreads, 0, s>>>(marks, m, direct ? nullptr : counts, map, inv, ctrl);
+    *launches += direct ? 1 : 2;
+    return cudaGetLastError();
+}
+
+// A's rows through the compaction map when it is used (grid-stride part of
+// the kernel that calls it); a row that held no entry when the map was made
+// is reported.
+__device__ __forceinline__ void remap_rows(const int32_t *Arow, int64_t nnz, const int32_t *map, int64_t m, int32_t *out,
+                                           Ctrl *ctrl) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nnz; i += stride) {
+        const int32_t r = Arow[i];
+        int32_t c = r >= 0 && r < m ? map[r] : -1;
+        if (c < 0) {
+            set_error(ctrl, SPG_ERR_INVALID, kDetailRowMap, i);
+            c = 0;
+        }
+        out[i] = c;
+    }
+}
+
+__global__ void k_row_remap(const int32_t *Arow, int64_t nnz, const int32_t *map, int64_t m, int32_t *out,
+                            Ctrl *ctrl) {
+    remap_rows(Arow, nnz, map, m, out, ctrl);
+}
+
+// Op_j = sum over stored B_kj of Z^A_k (Section 3.1), its bin, the bin
+// histogram and the total product count, with B's well-formedness checked on
+// the way (a bad pointer or row is reported and not followed) and A's rows
+// renumbered first where compaction applies.  Empty columns get nnz 0 here.
+//
+// A warp takes up to 32 columns, one per lane: runs of kDealRun neighbouring
+// columns (their pointers, Op and row entries share sectors), dealt through a
+// permutation of the runs (index times `mult` modulo their number, mult
+// coprime to it) so that the heavy columns of a skewed matrix, which sit
+// together (or, in R-MAT, at indices with few one bits), spread over the
+// CTAs.  A lane sums the Z^A_k of its own column up to kCountShort entries,
+// kCountUnroll gathers in flight; the longer columns of the CTA's eight warps
+// go on a list that the warps share, a warp per column.  A product of few
+// columns gives its warps fewer of them (`cols`), so that the gathers'
+// latency is spread over the chip.  Z^A_k is one 4-byte gather (a pair of
+// 8-byte column pointers kept L1's tag stage busy).  Dealing single columns,
+// flattening them 32 entries at a time with 64-bit warp scans and a 64-bit
+// division per column took 78 us for the very sparse product of 2^20 columns,
+// 47 us for R-MAT 2^18 and 28 us for 15013 columns of 23 entries; 48, 44
+// (53 with the renumbering of A) and 16 us so.
+constexpr int kCountThreads = 256;
+constexpr int kCountShort = 24;
+constexpr int kCountUnroll = 4;
+constexpr int kCountLong = 8;
+constexpr int kDealRun = 4;
+
+// x mod n for x < n^2 < 2^62, with inv = floor(2^64 / n) (n > 1): the quotient
+// from the high product is at most one short.
+__device__ __forceinline__ int64_t mod_by(unsigned long long x, unsigned long long n, unsigned long long inv) {
+    unsigned long long r = x - __umul64hi(x, inv) * n;
+    if (r >= n) r -= n;
+    return (int64_t)r;
+}
+
+__global__ void __launch_bounds__(kCountThreads) k_count_bin(CountArgs a, Ctrl *ctrl) {
     __shared__ unsigned long long s_hist[NBINS];
     __shared__ unsigned long long s_max[NBINS];
     __shared__ unsigned long long s_binprod[NBINS];
     __shared__ unsigned long long s_binb[NBINS];
     __shared__ unsigned long long s_prod, s_cap;
-    __shared__ int64_t s_op[32 * 32];  // per warp: the Op of its 32 columns (blockDim <= 1024)
+    __shared__ int64_t s_op[kCountThreads];    // Op of the CTA's columns
+    __shared__ int s_long[kCountThreads];      // columns (thread indices) of more than kCountShort entries
+    __shared__ int64_t s_lp[kCountThreads];    // their first entry
+    __shared__ int32_t s_ln[kCountThreads];    // and number of entries
+    __shared__ int s_nlong;
+    // what the row pass found: nothing here follows a malformed A
+    if (ctrl->err) return;
     if (threadIdx.x < NBINS) {
         s_hist[threadIdx.x] = 0;
         s_max[threadIdx.x] = 0;
@@ -57,102 +220,118 @@ __global__ void k_count_bin(const int64_t *__restrict__ Bcp, const int32_t *__re
         s_binb[threadIdx.x] = 0;
     }
     if (threadIdx.x == 0) s_prod = s_cap = 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    int64_t *wop = s_op + (threadIdx.x & ~31);
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const RowRule rows = row_rule((int64_t)ctrl->mrows, a.mA);
+    const int64_t t = effective_t(a.t, a.hmax, rows.m);
+    if (rows.compact) remap_rows(a.Arow, a.nnzA, a.rmap, a.mA, a.arow, ctrl);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned long long mine = 0, cap = 0;
-    for (int64_t g0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; g0 < nB; g0 += nwarps * 32) {
-        const int64_t g = g0 + lane;
-        const bool on = g < nB;
-        // mult < nB < 2^31 and g < nB: the product fits 63 bits
-        const int64_t j = on ? (int64_t)(((unsigned long long)g * (unsigned long long)mult) % (unsigned long long)nB)
-                             : 0;
-        int64_t p0 = 0, nb = 0;
+    const int64_t runs = (a.nB + kDealRun - 1) / kDealRun;
+    // runs per warp and CTA: a.cols / kDealRun, a power of two up to 8
+    const int rw = a.cols / kDealRun, rcta = rw * (kCountThreads / 32);
+    for (int64_t g0 = (int64_t)blockIdx.x * rcta; g0 < runs; g0 += (int64_t)gridDim.x * rcta) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_nlong = 0;
+        __syncthreads();
+        const int64_t g = lane < a.cols ? g0 + warp * rw + lane / kDealRun : runs;
+        const int64_t j = g < runs ? mod_by((unsigned long long)g * (unsigned long long)a.mult,
+                                            (unsigned long long)runs, a.inv) * kDealRun + lane % kDealRun
+                                   : a.nB;
+        const bool on = j < a.nB;
+        int64_t p0 = 0;
+        int nb = 0;
         if (on) {
-            p0 = Bcp[j];
-            nb = Bcp[j + 1] - p0;
+            p0 = a.Bcp[j];
+            const int64_t p1 = a.Bcp[j + 1];
+            if (a.validate && (p0 < 0 || p1 < p0 || p1 > a.nnzB || (j == 0 && p0 != 0) ||
+                               (j + 1 == a.nB && p1 != a.nnzB))) {
+                set_error(ctrl, SPG_ERR_INVALID, 2, j);
+                p0 = 0;
+            } else {
+                nb = (int)(p1 - p0);  // a column holds at most 2^31 - 1 distinct rows
+            }
         }
-        wop[lane] = 0;
-        // long columns: the whole warp, one column at a time
-        unsigned longs = __ballot_sync(0xffffffffu, nb > kCountLong);
-        while (longs) {
-            const int c = __ffs(longs) - 1;
-            longs &= longs - 1u;
-            const int64_t pc = __shfl_sync(0xffffffffu, p0, c);
-            const int64_t nc = __shfl_sync(0xffffffffu, nb, c);
+        if (nb > kCountShort) {
+            const int i = atomicAdd(&s_nlong, 1);
+            s_long[i] = threadIdx.x;
+            s_lp[i] = p0;
+            s_ln[i] = nb;
+        }
+        const int ns = nb > kCountShort ? 0 : nb;
+        int64_t s = 0;
+        for (int q0 = 0; q0 < ns; q0 += kCountUnroll) {
+            int32_t k[kCountUnroll];
+#pragma unroll
+            for (int u = 0; u < kCountUnroll; ++u) k[u] = q0 + u < ns ? a.Brow[p0 + q0 + u] : -1;
+#pragma unroll
+            for (int u = 0; u < kCountUnroll; ++u) {
+                if (q0 + u >= ns) continue;
+                if (a.validate && (k[u] < 0 || (int64_t)k[u] >= a.nA))
+                    set_error(ctrl, SPG_ERR_INVALID, 3, p0 + q0 + u);
+                else
+                    s += a.zlen[k[u]];
+            }
+        }
+        s_op[threadIdx.x] = s;
+        __syncthreads();
+        // long columns: one warp each, shared by the CTA's warps
+        const int nl = s_nlong;
+        for (int i = warp; i < nl; i += kCountThreads / 32) {
+            const int64_t pc = s_lp[i];
+            const int nc = s_ln[i];
             int64_t sz = 0;
-            for (int64_t p = pc + lane; p < pc + nc; p += 32) {
-                const int32_t k = Brow[p];
-                sz += Acp[k + 1] - Acp[k];
+            for (int q0 = lane; q0 < nc; q0 += 32 * kCountLong) {
+                int32_t k[kCountLong];
+#pragma unroll
+                for (int u = 0; u < kCountLong; ++u) {
+                    const int q = q0 + 32 * u;
+                    k[u] = q < nc ? a.Brow[pc + q] : -1;
+                    if (a.validate && q < nc && (k[u] < 0 || (int64_t)k[u] >= a.nA)) {
+                        set_error(ctrl, SPG_ERR_INVALID, 3, pc + q);
+                        k[u] = -1;
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < kCountLong; ++u)
+                    if (k[u] >= 0) sz += a.zlen[k[u]];
             }
 #pragma unroll
             for (int d = 16; d > 0; d >>= 1) sz += __shfl_xor_sync(0xffffffffu, sz, d);
-            if (lane == c) wop[c] = sz;
+            if (lane == 0) s_op[s_long[i]] = sz;
         }
-        // short columns: their entries as one flattened sequence
-        const int64_t ns = nb > kCountLong ? 0 : nb;
-        int64_t eincl = ns;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int64_t v = __shfl_up_sync(0xffffffffu, eincl, d);
-            if (lane >= d) eincl += v;
-        }
-        const int64_t eexcl = eincl - ns;
-        const int64_t E = __shfl_sync(0xffffffffu, eincl, 31);
-        __syncwarp();
-        for (int64_t e0 = 0; e0 < E; e0 += 32) {
-            const int64_t e = e0 + lane;
-            const int64_t q = e < E ? e : E - 1;
-            int c = 0;
-#pragma unroll
-            for (int step = 16; step > 0; step >>= 1) {
-                const int64_t ex = __shfl_sync(0xffffffffu, eexcl, c + step);
-                if (ex <= q) c += step;
-            }
-            const int64_t pc = __shfl_sync(0xffffffffu, p0, c);
-            const int64_t xc = __shfl_sync(0xffffffffu, eexcl, c);
-            int64_t z = 0;
-            if (e < E) {
-                const int32_t k = Brow[pc + (e - xc)];
-                z = Acp[k + 1] - Acp[k];
-            }
-            // owners are non-decreasing over the lanes: segmented inclusive sum
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const int64_t v = __shfl_up_sync(0xffffffffu, z, d);
-                const int oc = __shfl_up_sync(0xffffffffu, c, d);
-                if (lane >= d && oc == c) z += v;
-            }
-            const int cn = __shfl_down_sync(0xffffffffu, c, 1);
-            if (e < E && (lane == 31 || e + 1 >= E || cn != c)) wop[c] += z;
-            __syncwarp();
-        }
-        __syncwarp();
-        const int64_t s = wop[lane];
-    int b = -1;
+        __syncthreads();
+        s = s_op[threadIdx.x];
+        int b = -1;
         if (on) {
-            op[j] = s;
+            a.op[j] = s;
             mine += (unsigned long long)s;
-            cap += (unsigned long long)(s < mrows ? s : mrows);
-            b = bin_of(s, t, hmax, promote);
-            if (b == BIN_EMPTY) Ccp[j + 1] = 0;
+            cap += (unsigned long long)(s < rows.m ? s : rows.m);
+            b = bin_of(s, t, a.hmax, a.promote);
+            if (b == BIN_EMPTY) a.Ccp[j + 1] = 0;
         }
-        // per-bin statistics, one group of lanes per bin present
+        // per-bin statistics, one group of lanes per bin present; sums of 32
+        // values below 2^26 fit 32 bits (else 64-bit butterflies)
+        const bool small = __all_sync(0xffffffffu, s < (1 << 26) && nb < (1 << 26));
         unsigned pending = __ballot_sync(0xffffffffu, on);
         while (pending) {
             const int leader = __ffs(pending) - 1;
             const int bb = __shfl_sync(0xffffffffu, b, leader);
             const unsigned m = __ballot_sync(0xffffffffu, on && b == bb);
-            unsigned long long sm = (m >> lane) & 1u ? (unsigned long long)s : 0ull;
-            unsigned long long mx = sm;
-            unsigned long long nbs = (m >> lane) & 1u ? (unsigned long long)nb : 0ull;
+            const bool in = (m >> lane) & 1u;
+            unsigned long long sm, mx, nbs;
+            if (small) {
+                sm = __reduce_add_sync(0xffffffffu, in ? (unsigned)s : 0u);
+                mx = __reduce_max_sync(0xffffffffu, in ? (unsigned)s : 0u);
+                nbs = __reduce_add_sync(0xffffffffu, in ? (unsigned)nb : 0u);
+            } else {
+                sm = mx = in ? (unsigned long long)s : 0ull;
+                nbs = in ? (unsigned long long)nb : 0ull;
 #pragma unroll
-            for (int d = 16; d > 0; d >>= 1) {
-                sm += __shfl_xor_sync(0xffffffffu, sm, d);
-                nbs += __shfl_xor_sync(0xffffffffu, nbs, d);
-                const unsigned long long o = __shfl_xor_sync(0xffffffffu, mx, d);
-                if (o > mx) mx = o;
+                for (int d = 16; d > 0; d >>= 1) {
+                    sm += __shfl_xor_sync(0xffffffffu, sm, d);
+                    nbs += __shfl_xor_sync(0xffffffffu, nbs, d);
+                    const unsigned long long o = __shfl_xor_sync(0xffffffffu, mx, d);
+                    if (o > mx) mx = o;
+                }
             }
             if (lane == leader) {
                 atomicAdd(&s_hist[bb], (unsigned long long)__popc(m));
@@ -162,14 +341,16 @@ __global__ void k_count_bin(const int64_t *__restrict__ Bcp, const int32_t *__re
             }
             pending &= ~m;
         }
-        __syncwarp();
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) Ccp[0] = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.Ccp[0] = 0;
+        if (a.validate && a.nB == 0 && (a.Bcp[0] != 0 || a.nnzB != 0)) set_error(ctrl, SPG_ERR_INVALID, 2, 0);
+    }
     for (int d = 16; d > 0; d >>= 1) {
         mine += __shfl_xor_sync(0xffffffffu, mine, d);
         cap += __shfl_xor_sync(0xffffffffu, cap, d);
     }
-    if ((threadIdx.x & 31) == 0) {
+    if (lane == 0) {
         atomicAdd(&s_prod, mine);
         atomicAdd(&s_cap, cap);
     }
@@ -184,6 +365,20 @@ __global__ void k_count_bin(const int64_t *__restrict__ Bcp, const int32_t *__re
         atomicAdd(&ctrl->products, s_prod);
         atomicAdd(&ctrl->capsum, s_cap);
     }
+}
+
+cudaError_t launch_count_bin(const CountArgs &args, int sms, Ctrl *ctrl, cudaStream_t s) {
+    CountArgs a = args;
+    const int64_t runs = ceil_div(a.nB, kDealRun);
+    a.mult = column_deal_mult(runs);
+    // floor(2^64 / runs); one run only ever asks for 0 mod 1
+    a.inv = runs > 1 ? (unsigned long long)(((unsigned __int128)1 << 64) / (unsigned __int128)runs) : 0;
+    // eight warps a CTA; at least four CTAs per SM before a warp takes more
+    a.cols = kDealRun;
+    while (a.cols < 32 && ceil_div(a.nB, 8 * a.cols) > 4 * (int64_t)sms) a.cols *= 2;
+    const int g = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(a.nB, 8 * a.cols), 16 * (int64_t)sms));
+    k_count_bin<<<g, kCountThreads, 0, s>>>(a, ctrl);
+    return cudaGetLastError();
 }
 
 int64_t column_deal_mult(int64_t n) {
@@ -318,27 +513,71 @@ cudaError_t launch_slot_copy(int64_t nB, int64_t nnzC, const int64_t *Ccp, const
 
 int64_t copy_tile_count(int64_t n) { return n / kCopyTile + 2; }
 
-// Column ids into per-bin lists at off[bin] (each block reserves its slots
-// with one global atomic per bin, so columns of a bin stay roughly in
-// ascending order within a block's tile).
-__global__ void k_bin_scatter(const int64_t *__restrict__ op, int64_t nB, int64_t t, int64_t hmax, int promote,
-                              BinOffsets off, int32_t *__restrict__ bin_cols, Ctrl *ctrl) {
+// Column ids into per-bin lists (each block reserves its slots with one
+// global atomic per bin, so columns of a bin stay roughly in ascending order
+// within a block's tile).  The lists start at the running sums of the bins'
+// counts, taken from the control block, so nothing of it waits for the host;
+// block 0 then writes the control block to the host's mirror (the host reads
+// its counts and errors, not the scatter cursors this kernel moves).
+constexpr int kScatterThreads = 256;
+constexpr int kScatterItems = 4;  // columns per thread: fewer blocks on the bins' cursors
+
+__global__ void __launch_bounds__(kScatterThreads) k_bin_scatter(const int64_t *__restrict__ op, int64_t nB,
+                                                                int64_t tcfg, int64_t hmax, int promote, int64_t mA,
+                                                                int32_t *__restrict__ bin_cols, Ctrl *ctrl,
+                                                                unsigned char *host) {
     __shared__ unsigned int s_cnt[NBINS];
     __shared__ unsigned long long s_base[NBINS];
+    if (host && blockIdx.x == 0)
+        for (int i = threadIdx.x; i < (int)(sizeof(Ctrl) / 8); i += kScatterThreads)
+            reinterpret_cast<unsigned long long *>(host)[i] = reinterpret_cast<const unsigned long long *>(ctrl)[i];
+    if (ctrl->err || !bin_cols) return;  // Op is not there for a malformed product
     if (threadIdx.x < NBINS) s_cnt[threadIdx.x] = 0;
     __syncthreads();
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int b = -1;
-    unsigned r = 0;
-    if (j < nB) {
-        b = bin_of(op[j], t, hmax, promote);
-        if (b != BIN_EMPTY) r = atomicAdd(&s_cnt[b], 1u);
+    const int64_t t = effective_t(tcfg, hmax, row_rule((int64_t)ctrl->mrows, mA).m);
+    const int lane = threadIdx.x & 31;
+    const int64_t j0 = (int64_t)blockIdx.x * (kScatterThreads * kScatterItems) + threadIdx.x;
+    int b[kScatterItems];
+    unsigned r[kScatterItems];
+#pragma unroll
+    for (int u = 0; u < kScatterItems; ++u) {
+        const int64_t j = j0 + u * kScatterThreads;
+        b[u] = j < nB ? bin_of(op[j], t, hmax, promote) : BIN_EMPTY;
+        r[u] = 0;
+    }
+#pragma unroll
+    for (int u = 0; u < kScatterItems; ++u) {
+        unsigned pending = __ballot_sync(0xffffffffu, b[u] != BIN_EMPTY);
+        while (pending) {
+            const int leader = __ffs(pending) - 1;
+            const int bb = __shfl_sync(0xffffffffu, b[u], leader);
+            const unsigned m = __ballot_sync(0xffffffffu, b[u] == bb);
+            unsigned at = 0;
+            if (lane == leader) at = atomicAdd(&s_cnt[bb], (unsigned)__popc(m));
+            at = __shfl_sync(0xffffffffu, at, leader);
+            if (b[u] == bb) r[u] = at + __popc(m & ((1u << lane) - 1u));
+            pending &= ~m;
+        }
     }
     __syncthreads();
-    if (threadIdx.x < NBINS && s_cnt[threadIdx.x])
-        s_base[threadIdx.x] = atomicAdd(&ctrl->fill[threadIdx.x], (unsigned long long)s_cnt[threadIdx.x]);
+    if (threadIdx.x < NBINS && s_cnt[threadIdx.x]) {
+        unsigned long long off = 0;
+        for (int i = BIN_EMPTY + 1; i < (int)threadIdx.x; ++i) off += ctrl->hist[i];
+        s_base[threadIdx.x] = off + atomicAdd(&ctrl->fill[threadIdx.x], (unsigned long long)s_cnt[threadIdx.x]);
+    }
     __syncthreads();
-    if (b > BIN_EMPTY) bin_cols[off.v[b] + (int64_t)s_base[b] + r] = (int32_t)j;
+#pragma unroll
+    for (int u = 0; u < kScatterItems; ++u)
+        if (b[u] != BIN_EMPTY) bin_cols[(int64_t)s_base[b[u]] + r[u]] = (int32_t)(j0 + u * kScatterThreads);
+}
+
+cudaError_t launch_bin_scatter(const CountArgs &a, int32_t *bin_cols, Ctrl *ctrl, unsigned char *host,
+                               cudaStream_t s) {
+    static_assert(sizeof(Ctrl) % 8 == 0, "the control block is copied in 8-byte words");
+    const int64_t g = bin_cols ? std::max<int64_t>(1, ceil_div(a.nB, kScatterThreads * kScatterItems)) : 1;
+    k_bin_scatter<<<(unsigned)g, kScatterThreads, 0, s>>>(a.op, a.nB, a.t, a.hmax, a.promote, a.mA, bin_cols, ctrl,
+                                                          host);
+    return cudaGetLastError();
 }
 
 // ----------------------------------------------------------- int64 scan
@@ -400,7 +639,15 @@ __global__ void k_scan_sums(int64_t *sums, int64_t ntiles) {
     }
 }
 
-__global__ void k_scan_apply(int64_t *__restrict__ x, int64_t n, const int64_t *__restrict__ sums) {
+// summed: sums holds the exclusive prefix of the tiles' sums, else the sums
+// themselves, which the CTA adds up to its own tile (one launch fewer, for as
+// many tiles as kScanDirect).  With `host`, the last tile's CTA writes the
+// scan's last value and the control block to the host's mirror.
+constexpr int64_t kScanDirect = 4096;
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_apply(int64_t *__restrict__ x, int64_t n,
+                                                            const int64_t *__restrict__ sums, int summed,
+                                                            const Ctrl *ctrl, unsigned char *host) {
     __shared__ int64_t s_warp[32];
     const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
     int64_t v[kScanItems];
@@ -411,62 +658,47 @@ __global__ void k_scan_apply(int64_t *__restrict__ x, int64_t n, const int64_t *
         v[i] = e < n ? x[e] : 0;
         s += v[i];
     }
+    int64_t before = 0;
+    if (summed) {
+        before = sums[blockIdx.x];
+    } else if (blockIdx.x > 0) {  // uniform over the CTA
+        int64_t part = 0;
+        for (int64_t i = threadIdx.x; i < blockIdx.x; i += kScanThreads) part += sums[i];
+        block_incl_scan_i64(part, s_warp, before);
+    }
     int64_t total;
     int64_t incl = block_incl_scan_i64(s, s_warp, total);
-    int64_t run = sums[blockIdx.x] + incl - s;
+    int64_t run = before + incl - s;
 #pragma unroll
     for (int i = 0; i < kScanItems; ++i) {
         int64_t e = base + i;
         run += v[i];
         if (e < n) x[e] = run;
     }
+    if (host && blockIdx.x + 1 == gridDim.x) {
+        if (threadIdx.x == 0) *reinterpret_cast<int64_t *>(host) = before + total;
+        for (int i = threadIdx.x; i < (int)(sizeof(Ctrl) / 8); i += kScanThreads)
+            reinterpret_cast<unsigned long long *>(host)[1 + i] = reinterpret_cast<const unsigned long long *>(ctrl)[i];
+    }
 }
 
-cudaError_t launch_inclusive_scan(int64_t *x, int64_t n, int64_t *tile_sums, cudaStream_t s) {
+int scan_launches(int64_t n) {
+    const int64_t ntiles = scan_tile_count(n);
+    return n <= 0 ? 0 : ntiles == 1 ? 1 : ntiles <= kScanDirect ? 2 : 3;
+}
+
+cudaError_t launch_inclusive_scan(int64_t *x, int64_t n, int64_t *tile_sums, cudaStream_t s, const Ctrl *ctrl,
+                                  unsigned char *host) {
     if (n <= 0) return cudaSuccess;
     const int64_t ntiles = ceil_div(n, kScanTile);
-    k_scan_tiles<<<(unsigned)ntiles, kScanThreads, 0, s>>>(x, n, tile_sums);
-    k_scan_sums<<<1, 1024, 0, s>>>(tile_sums, ntiles);
-    k_scan_apply<<<(unsigned)ntiles, kScanThreads, 0, s>>>(x, n, tile_sums);
+    const bool summed = ntiles > kScanDirect;
+    if (ntiles > 1) k_scan_tiles<<<(unsigned)ntiles, kScanThreads, 0, s>>>(x, n, tile_sums);
+    if (summed) k_scan_sums<<<1, 1024, 0, s>>>(tile_sums, ntiles);
+    k_scan_apply<<<(unsigned)ntiles, kScanThreads, 0, s>>>(x, n, tile_sums, summed ? 1 : 0, ctrl, host);
     return cudaGetLastError();
 }
 
 int64_t scan_tile_count(int64_t n) { return n <= 0 ? 1 : ceil_div(n, kScanTile); }
-
-
-
-// ------------------------------------------------------- row compaction
-__global__ void k_row_mark(const int32_t *Arow, int64_t nnz, int64_t m, int64_t *mark) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nnz; i += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t r = Arow[i];
-        if (r >= 0 && r < m) mark[r] = 1;
-    }
-}
-
-__global__ void k_row_map(const int64_t *incl, int64_t m, int32_t *map, int32_t *inv) {
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < m; r += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t before = r > 0 ? incl[r - 1] : 0;
-        if (incl[r] != before) {
-            map[r] = (int32_t)before;
-            inv[before] = (int32_t)r;
-        } else {
-            map[r] = -1;
-        }
-    }
-}
-
-__global__ void k_row_remap(const int32_t *Arow, int64_t nnz, const int32_t *map, int64_t m, int32_t *out,
-                            Ctrl *ctrl) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nnz; i += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t r = Arow[i];
-        int32_t c = r >= 0 && r < m ? map[r] : -1;
-        if (c < 0) {
-            set_error(ctrl, SPG_ERR_INVALID, kDetailRowMap, i);
-            c = 0;
-        }
-        out[i] = c;
-    }
-}
 
 // ------------------------------------------------------------ readback
 namespace {
@@ -481,6 +713,12 @@ constexpr int kMaxDevices = 64;
 thread_local Mirror t_mirror[kMaxDevices];
 
 }  // namespace
+
+Mirror *thread_mirror() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+    return &t_mirror[dev];
+}
 
 Mirror::~Mirror() {
     if (host) cudaFreeHost(host);
@@ -505,12 +743,7 @@ cudaError_t Mirror::reserve(size_t need) {
 cudaError_t readback(Mirror *mp, void *dst0, const void *src0, size_t n0, void *dst1, const void *src1, size_t n1,
                      cudaStream_t s) {
     cudaError_t e;
-    if (!mp) {
-        int dev = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-        if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-        mp = &t_mirror[dev];
-    }
+    if (!mp && !(mp = thread_mirror())) return cudaErrorInvalidDevice;
     Mirror &m = *mp;
     const size_t off1 = (n0 + 15) & ~size_t(15);
     if ((e = m.reserve(off1 + n1)) != cudaSuccess) return e;

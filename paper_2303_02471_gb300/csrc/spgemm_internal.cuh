@@ -34,19 +34,30 @@ __host__ __device__ constexpr int warp_bin_R(int b) {
 __host__ __device__ constexpr int warp_bin_opmax(int b) { return warp_bin_G(b) * warp_bin_R(b); }
 __host__ __device__ constexpr int64_t cta_bin_opmax(int c) { return 512LL << c; }
 
+// Smallest e with 2^e >= v, for v > 1.
+__host__ __device__ inline int log2_ceil(uint32_t v) {
+#ifdef __CUDA_ARCH__
+    return 32 - __clz((int)(v - 1));
+#else
+    return 32 - __builtin_clz(v - 1);
+#endif
+}
+static_assert(warp_bin_opmax(0) == 8 && warp_bin_opmax(kNumWarpBins - 1) == 8 << (kNumWarpBins - 1) &&
+                  cta_bin_opmax(0) == 512,
+              "bin_of takes the bins' limits for powers of two");
+
 // Bin of a column with Op_j = op under threshold t and CTA-hash limit; a
 // column of a lane-group bin moves `promote` group bins up (more lanes and
 // table slots per column), at most to the last group bin.
 __host__ __device__ inline int bin_of(int64_t op, int64_t t, int64_t hash_cta_max, int promote = 0) {
     if (op <= 0) return BIN_EMPTY;
     if (op >= t) return BIN_DENSE;
-    for (int b = 0; b < kNumWarpBins; ++b)
-        if (op <= warp_bin_opmax(b))
-            return BIN_WARP0 + (b + promote < kNumWarpBins ? b + promote : kNumWarpBins - 1);
-    if (op <= hash_cta_max) {
-        for (int c = 0; c < kNumCtaBins; ++c)
-            if (op <= cta_bin_opmax(c)) return BIN_CTA0 + c;
+    // the bins' limits are powers of two: 8 << b, then 512 << c
+    if (op <= warp_bin_opmax(kNumWarpBins - 1)) {
+        const int b = op <= 8 ? 0 : log2_ceil((uint32_t)op) - 3;
+        return BIN_WARP0 + (b + promote < kNumWarpBins ? b + promote : kNumWarpBins - 1);
     }
+    if (op <= hash_cta_max && op <= cta_bin_opmax(kNumCtaBins - 1)) return BIN_CTA0 + log2_ceil((uint32_t)op) - 9;
     return BIN_GLOBAL;
 }
 
@@ -67,7 +78,8 @@ struct Ctrl {
     unsigned long long binnnzb[NBINS];  // sum of nnz(B_j) per bin
     unsigned long long products;        // sum_j Op_j
     unsigned long long capsum;          // sum_j min(Op_j, rows): the single pass's slots
-    unsigned long long pad[2];
+    unsigned long long mrows;           // rows of A that hold entries
+    unsigned long long pad;
 };
 
 // Code for a column whose numeric count disagrees with the symbolic one
