@@ -308,6 +308,14 @@ spg_status spgemm_backward(spg_plan *plan, const spg_csc *A, const spg_csc *B,
  *   nnzC (host), and returns a plan whose slots hold C.  The plan also serves
  *   spgemm_numeric (which recomputes C from the A and B it is given, into the
  *   caller's buffers), spgemm_backward and the plan queries.  Synchronises.
+ * spgemm_single_pass_begin, spgemm_single_pass_finish: spgemm_single_pass in
+ *   two calls, for a caller that allocates the slots once their size is known
+ *   instead of asking for it with a preparation of its own.  begin prepares in
+ *   `workspace` (spgemm_workspace_size bytes with cfg->dense_cache_bytes = 0)
+ *   and returns the plan and the bytes of the slots; finish, once per plan and
+ *   with the same A and B, writes C into `slots` (device, 256-byte aligned,
+ *   kept by the caller while the plan is used), C_colptr and nnzC.  A plan
+ *   whose finish failed serves only spg_plan_destroy.  Both synchronise.
  * spgemm_single_pass_copy: C's rows (device int32[nnzC]) and values (device,
  *   plan dtype) from the plan's slots, in order; asynchronous.  The values are
  *   those of the A and B given to spgemm_single_pass.
@@ -325,6 +333,15 @@ spg_status spgemm_single_pass(spg_handle *handle, const spg_csc *A,
                               void *workspace, size_t ws_bytes,
                               int64_t *C_colptr, int64_t *nnzC,
                               spg_plan **plan, spg_stream stream);
+spg_status spgemm_single_pass_begin(spg_handle *handle, const spg_csc *A,
+                                    const spg_csc *B, const spg_config *cfg,
+                                    void *workspace, size_t ws_bytes,
+                                    int64_t *C_colptr, size_t *slot_bytes,
+                                    spg_plan **plan, spg_stream stream);
+spg_status spgemm_single_pass_finish(spg_plan *plan, const spg_csc *A,
+                                     const spg_csc *B, void *slots,
+                                     size_t slot_bytes, int64_t *C_colptr,
+                                     int64_t *nnzC, spg_stream stream);
 spg_status spgemm_single_pass_copy(spg_plan *plan, const int64_t *C_colptr,
                                    int32_t *C_rowidx, void *C_values,
                                    spg_stream stream);

@@ -61,6 +61,9 @@ SIGNATURES = {
                                       vp]),
     "spgemm_single_pass": (i32, [vp, vp, vp, vp, vp, ctypes.c_size_t, vp, ctypes.POINTER(i64),
                                  ctypes.POINTER(vp), vp]),
+    "spgemm_single_pass_begin": (i32, [vp, vp, vp, vp, vp, ctypes.c_size_t, vp, ctypes.POINTER(ctypes.c_size_t),
+                                       ctypes.POINTER(vp), vp]),
+    "spgemm_single_pass_finish": (i32, [vp, vp, vp, vp, ctypes.c_size_t, vp, ctypes.POINTER(i64), vp]),
     "spgemm_single_pass_copy": (i32, [vp, vp, vp, vp, vp]),
     "spgemm_backward": (i32, [vp, vp, vp, vp, vp, vp, vp, vp, vp]),
     "spgemm_csr_workspace_size": (i32, [vp, vp, vp, ctypes.POINTER(ctypes.c_size_t)]),

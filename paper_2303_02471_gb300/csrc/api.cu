@@ -155,10 +155,11 @@ struct spg_plan {
     // lane-group bins worked by the ESC accumulator (and their tile shapes)
     bool esc[NBINS] = {};
     EscShape esc_shape_of[NBINS];
-    // single pass: the columns' slots (offsets, rows, values) after the
-    // regular layout, sum of the slot sizes
+    // single pass: the columns' slots (offsets, rows, values) in a buffer of
+    // their own or after the regular layout, sum of the slot sizes
     bool single = false;
-    size_t soff_at = 0, srow_at = 0, sval_at = 0, tcol_at = 0, slots_total = 0;
+    unsigned char *slots = nullptr;
+    size_t soff_at = 0, srow_at = 0, sval_at = 0, tcol_at = 0, slot_bytes = 0;
     int64_t capsum = 0;
 
     ~spg_plan() {
@@ -337,12 +338,12 @@ spg_status spg_destroy(spg_handle *handle) {
     return SPG_OK;
 }
 
-// Slots of the single pass after the regular layout: offsets int64[nB + 1],
-// rows int32[capsum], values[capsum], and the copy's first column of every
-// tile of C's positions (nnz(C) <= capsum).
+// Slots of the single pass: offsets int64[nB + 1], rows int32[capsum],
+// values[capsum], and the copy's first column of every tile of C's positions
+// (nnz(C) <= capsum).
 static void slot_layout(spg_plan *P) {
     const size_t w = P->dtype == SPG_F64 ? 8 : 4;
-    size_t off = align256(P->L.total);
+    size_t off = 0;
     P->soff_at = off;
     off = align256(off + (size_t)(P->nB + 1) * 8);
     P->srow_at = off;
@@ -351,7 +352,7 @@ static void slot_layout(spg_plan *P) {
     off = align256(off + (size_t)P->capsum * w);
     P->tcol_at = off;
     off = align256(off + (size_t)copy_tile_count(P->capsum) * 4);
-    P->slots_total = off;
+    P->slot_bytes = off;
 }
 
 // Everything before the accumulators, shared by the symbolic phase and the
@@ -616,34 +617,44 @@ spg_status spgemm_single_pass_size(spg_handle *handle, const spg_csc *A, const s
                       &P)) != SPG_OK)
         return st;
     slot_layout(P);
-    *bytes = P->slots_total;
+    *bytes = align256(P->L.total) + P->slot_bytes;
     delete P;
     return SPG_OK;
 }
 
-spg_status spgemm_single_pass(spg_handle *handle, const spg_csc *A, const spg_csc *B, const spg_config *cfg,
-                              void *workspace, size_t ws_bytes, int64_t *C_colptr, int64_t *nnzC,
-                              spg_plan **plan_out, spg_stream stream) {
+spg_status spgemm_single_pass_begin(spg_handle *handle, const spg_csc *A, const spg_csc *B, const spg_config *cfg,
+                                    void *workspace, size_t ws_bytes, int64_t *C_colptr, size_t *slot_bytes,
+                                    spg_plan **plan_out, spg_stream stream) {
     if (plan_out) *plan_out = nullptr;
-    if (!C_colptr || !nnzC || !plan_out) return SPG_ERR_INVALID;
+    if (!C_colptr || !slot_bytes || !plan_out) return SPG_ERR_INVALID;
     spg_status st = check_pair(A, B, true);
     if (st != SPG_OK) return st;
     spg_config c = normalized(cfg);
     if ((st = check_config(c)) != SPG_OK) return st;
-    c.dense_cache_bytes = 0;
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    c.dense_cache_bytes = 0;  // nothing is kept between phases
     spg_plan *P = nullptr;
-    if ((st = prepare(handle, A, B, c, workspace, ws_bytes, C_colptr, s, true, &P)) != SPG_OK) return st;
+    if ((st = prepare(handle, A, B, c, workspace, ws_bytes, C_colptr, reinterpret_cast<cudaStream_t>(stream), true,
+                      &P)) != SPG_OK)
+        return st;
     slot_layout(P);
-    if (ws_bytes < P->slots_total) { delete P; return SPG_ERR_WORKSPACE; }
-    P->single = true;
-    Ctrl *ctrl = P->ctrl();
-    int64_t *soff = reinterpret_cast<int64_t *>(P->ws + P->soff_at);
+    *slot_bytes = P->slot_bytes;
+    *plan_out = P;
+    return SPG_OK;
+}
 
-#define CK(expr)                                                      \
-    do {                                                              \
-        cudaError_t e_ = (expr);                                      \
-        if (e_ != cudaSuccess) { delete P; return SPG_ERR_CUDA; }     \
+spg_status spgemm_single_pass_finish(spg_plan *P, const spg_csc *A, const spg_csc *B, void *slots, size_t slot_bytes,
+                                     int64_t *C_colptr, int64_t *nnzC, spg_stream stream) {
+    spg_status st = check_plan_operands(P, A, B);
+    if (st != SPG_OK) return st;
+    if (!C_colptr || !nnzC || P->num_geo_ready || P->slot_bytes == 0) return SPG_ERR_INVALID;
+    if (!slots || (reinterpret_cast<uintptr_t>(slots) & 255) || slot_bytes < P->slot_bytes) return SPG_ERR_WORKSPACE;
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    P->slots = static_cast<unsigned char *>(slots);
+    int64_t *soff = reinterpret_cast<int64_t *>(P->slots + P->soff_at);
+
+#define CK(expr)                                       \
+    do {                                               \
+        if ((expr) != cudaSuccess) return SPG_ERR_CUDA; \
     } while (0)
 
     // slot offsets: an exclusive scan of min(Op_j, rows)
@@ -658,22 +669,43 @@ spg_status spgemm_single_pass(spg_handle *handle, const spg_csc *A, const spg_cs
     for (int b = 1; b < NBINS; ++b) {
         if (!P->host.hist[b]) continue;
         const int64_t bound = std::min<int64_t>((int64_t)P->host.maxop[b], P->mC);
-        P->num_geo[b] = numeric_geometry(b, (int64_t)P->host.hist[b], P->mC, c.cta_threads, P->dev.sms,
-                                         P->dev.smem_optin, bound, P->dtype, c.table_slots_pct, P->L.scratch_ctas);
+        P->num_geo[b] = numeric_geometry(b, (int64_t)P->host.hist[b], P->mC, P->cfg.cta_threads, P->dev.sms,
+                                         P->dev.smem_optin, bound, P->dtype, P->cfg.table_slots_pct,
+                                         P->L.scratch_ctas);
     }
     P->num_geo_ready = true;
     Operands o{A->colptr, P->compact ? P->arow() : A->rowidx, A->values, B->colptr, B->rowidx, B->values,
                P->compact ? P->rinv() : nullptr};
-    st = run_numeric(P, o, soff, C_colptr, reinterpret_cast<int32_t *>(P->ws + P->srow_at), P->ws + P->sval_at, s);
-    if (st != SPG_OK) { delete P; return st; }
+    st = run_numeric(P, o, soff, C_colptr, reinterpret_cast<int32_t *>(P->slots + P->srow_at), P->slots + P->sval_at, s);
+    if (st != SPG_OK) return st;
     CK(P->scan_and_read(C_colptr, s));
 #undef CK
-    if (P->host.err) { st = (spg_status)P->host.err; delete P; return st; }
+    if (P->host.err) return (spg_status)P->host.err;
     // the preparation, slot caps and their scan, the bins, the scan with the
     // control read
     P->sym_launches += (P->nB > 0 ? 1 + scan_launches(P->nB) : 0) + P->nonempty_bins() +
                        std::max(1, scan_launches(P->nB));
+    P->single = true;
     *nnzC = P->nnzC;
+    return SPG_OK;
+}
+
+spg_status spgemm_single_pass(spg_handle *handle, const spg_csc *A, const spg_csc *B, const spg_config *cfg,
+                              void *workspace, size_t ws_bytes, int64_t *C_colptr, int64_t *nnzC,
+                              spg_plan **plan_out, spg_stream stream) {
+    if (plan_out) *plan_out = nullptr;
+    if (!C_colptr || !nnzC || !plan_out) return SPG_ERR_INVALID;
+    size_t slot_bytes = 0;
+    spg_plan *P = nullptr;
+    spg_status st =
+        spgemm_single_pass_begin(handle, A, B, cfg, workspace, ws_bytes, C_colptr, &slot_bytes, &P, stream);
+    if (st != SPG_OK) return st;
+    // the slots follow the regular layout
+    const size_t at = align256(P->L.total);
+    st = ws_bytes < at + slot_bytes ? SPG_ERR_WORKSPACE
+                                    : spgemm_single_pass_finish(P, A, B, P->ws + at, ws_bytes - at, C_colptr, nnzC,
+                                                                stream);
+    if (st != SPG_OK) { delete P; return st; }
     *plan_out = P;
     return SPG_OK;
 }
@@ -682,10 +714,10 @@ spg_status spgemm_single_pass_copy(spg_plan *P, const int64_t *C_colptr, int32_t
                                    spg_stream stream) {
     if (!P || !P->single || !C_colptr || (P->nnzC > 0 && (!C_rowidx || !C_values))) return SPG_ERR_INVALID;
     const int w = P->dtype == SPG_F64 ? 8 : 4;
-    return cuda_status(launch_slot_copy(P->nB, P->nnzC, C_colptr, reinterpret_cast<const int64_t *>(P->ws + P->soff_at),
-                                        reinterpret_cast<int32_t *>(P->ws + P->tcol_at),
-                                        reinterpret_cast<const int32_t *>(P->ws + P->srow_at),
-                                        P->ws + P->sval_at, C_rowidx, C_values, w, P->dev.sms,
+    return cuda_status(launch_slot_copy(P->nB, P->nnzC, C_colptr, reinterpret_cast<const int64_t *>(P->slots + P->soff_at),
+                                        reinterpret_cast<int32_t *>(P->slots + P->tcol_at),
+                                        reinterpret_cast<const int32_t *>(P->slots + P->srow_at),
+                                        P->slots + P->sval_at, C_rowidx, C_values, w, P->dev.sms,
                                         reinterpret_cast<cudaStream_t>(stream)));
 }
 

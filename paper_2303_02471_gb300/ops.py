@@ -215,6 +215,7 @@ class Plan:
         self._h = handle
         self._lib_handle = lib_handle  # kept alive while the plan is
         self.workspace = workspace
+        self.slots = None  # single pass: C's columns, until they are copied
         self.shape = (A.nrows, B.ncols)
         self.dtype = A.dtype
         self.colptr = colptr
@@ -357,16 +358,29 @@ def spgemm_single_pass(A: CscMatrix, B: CscMatrix, config: Optional[Config] = No
     config = config or Config()
     hd = lib_handle if lib_handle is not None else handle(A.device)
     cA, cB = _csc(A), _csc(B, A.dtype)
-    if workspace is None:  # a workspace given is checked by the call itself
-        need = single_pass_workspace_size(A, B, config, hd)
-        workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=A.device)
     colptr = torch.empty(B.ncols + 1, dtype=torch.int64, device=A.device)
     nnz = ctypes.c_int64()
     h = ctypes.c_void_p()
-    N.check(N.lib().spgemm_single_pass(hd.ptr, ctypes.byref(cA), ctypes.byref(cB), ctypes.byref(config.native()),
-                                       _ptr(workspace), workspace.numel(), _ptr(colptr), ctypes.byref(nnz),
-                                       ctypes.byref(h), _stream()), "spgemm_single_pass")
-    plan = Plan(h, workspace, A, B, colptr, nnz.value, config, hd)
+    if workspace is None:
+        # the slots are allocated between the preparation and the pass
+        single = replace(config, dense_cache_bytes=0)
+        workspace = torch.empty(max(workspace_size(A, B, single), 256), dtype=torch.uint8, device=A.device)
+        need = ctypes.c_size_t()
+        N.check(N.lib().spgemm_single_pass_begin(hd.ptr, ctypes.byref(cA), ctypes.byref(cB),
+                                                 ctypes.byref(single.native()), _ptr(workspace), workspace.numel(),
+                                                 _ptr(colptr), ctypes.byref(need), ctypes.byref(h), _stream()),
+                "spgemm_single_pass_begin")
+        plan = Plan(h, workspace, A, B, colptr, 0, config, hd)
+        plan.slots = torch.empty(max(need.value, 256), dtype=torch.uint8, device=A.device)
+        N.check(N.lib().spgemm_single_pass_finish(h, ctypes.byref(cA), ctypes.byref(cB), _ptr(plan.slots),
+                                                  plan.slots.numel(), _ptr(colptr), ctypes.byref(nnz), _stream()),
+                "spgemm_single_pass_finish")
+        plan.nnz = nnz.value
+    else:  # checked by the call itself
+        N.check(N.lib().spgemm_single_pass(hd.ptr, ctypes.byref(cA), ctypes.byref(cB), ctypes.byref(config.native()),
+                                           _ptr(workspace), workspace.numel(), _ptr(colptr), ctypes.byref(nnz),
+                                           ctypes.byref(h), _stream()), "spgemm_single_pass")
+        plan = Plan(h, workspace, A, B, colptr, nnz.value, config, hd)
     rowidx = torch.empty(nnz.value, dtype=torch.int32, device=A.device)
     values = torch.empty(nnz.value, dtype=A.dtype, device=A.device)
     N.check(N.lib().spgemm_single_pass_copy(plan.handle, _ptr(colptr), _ptr(rowidx), _ptr(values), _stream()),
