@@ -152,9 +152,8 @@ struct spg_plan {
     // created on first use
     spg_handle *h = nullptr;
     SideStreams own;
-    // lane-group bins worked by the ESC accumulator (and their tile shapes)
+    // lane-group bins whose values the ESC accumulator works
     bool esc[NBINS] = {};
-    EscShape esc_shape_of[NBINS];
     // single pass: the columns' slots (offsets, rows, values) in a buffer of
     // their own or after the regular layout, sum of the slot sizes
     bool single = false;
@@ -428,11 +427,9 @@ static spg_status prepare(spg_handle *handle, const spg_csc *A, const spg_csc *B
         P->off.v[b + 1] = P->off.v[b] + n;
     }
 #undef CK
-    // the numeric phase (and the single pass) take ESC unless hash tables
-    // were asked for; the symbolic phase counts with ESC when asked, and by
-    // default in the bins that ESC sorts by rank (sym_bin)
+    // the light columns take ESC unless hash tables were asked for
     if (c.small_accumulator != SPG_ACC_HASH)
-        for (int b = BIN_WARP0; b < BIN_CTA0; ++b) P->esc[b] = esc_shape(b, P->mC, P->esc_shape_of[b]);
+        for (int b = BIN_WARP0; b < BIN_CTA0; ++b) P->esc[b] = true;
     // A's checks and row marks, the row index, Op counting, the scatter with
     // the control read
     P->sym_launches = 3 + launches;
@@ -460,7 +457,8 @@ spg_status spgemm_symbolic(spg_handle *handle, const spg_csc *A, const spg_csc *
         if (e_ != cudaSuccess) { delete P; return SPG_ERR_CUDA; }     \
     } while (0)
 
-    Operands o{A->colptr, P->compact ? P->arow() : A->rowidx, nullptr, B->colptr, B->rowidx, nullptr};
+    Operands o{A->colptr, P->compact ? P->arow() : A->rowidx, nullptr, B->colptr, B->rowidx, nullptr, nullptr,
+               std::max(A->nnz, B->nnz)};
     // as in the numeric phase: beside a dense bin, the lane-group bins (shared
     // memory only) run on the side streams, launched after the dense kernel
     bool groups = false;
@@ -471,13 +469,14 @@ spg_status spgemm_symbolic(spg_handle *handle, const spg_csc *A, const spg_csc *
         CK(cudaEventRecord(P->ss().fork, s));
     }
     auto sym_bin = [&](int b, cudaStream_t sb) {
-        // counting by rank (no sort, no compress) beat the hash tables on
-        // GB300; counting through the radix sort did not
-        const bool esc_counts = c.small_accumulator == SPG_ACC_ESC ||
-                                (c.small_accumulator == SPG_ACC_AUTO && P->esc_shape_of[b].rank != kEscRadix);
+        // counting with ESC beats the hash tables where a filter of the rows
+        // spares most columns the sort (bins of up to 64 products: 227 against
+        // 560 us for the very sparse product of 2^20 columns), not in the
+        // larger bins (35 against 48 us for 25000 columns of 129..256)
+        const bool esc_counts = c.small_accumulator == SPG_ACC_ESC || warp_bin_opmax(b - BIN_WARP0) <= 64;
         if (P->esc[b] && esc_counts)
-            return launch_esc_bin(P->task(b), o, C_colptr, C_colptr, nullptr, nullptr, false, P->dtype,
-                                  P->esc_shape_of[b], P->dev.sms, sb);
+            return launch_esc_bin(P->task(b), o, C_colptr, C_colptr, nullptr, nullptr, false, P->dtype, P->dev.sms,
+                                  sb);
         // the symbolic CTA kernels carry no values: CTAs of up to 256 threads,
         // several per SM, overlap one another's barriers (measured faster)
         Geo g = symbolic_geometry(b, (int64_t)P->host.hist[b], P->mC, std::min(c.cta_threads, kSymCtaThreads),
@@ -547,7 +546,7 @@ static spg_status run_numeric(spg_plan *P, const Operands &o, const int64_t *bas
         t.cnt_out = cnt_out;
         if (cnt_out) t.cache_cols = 0;  // no symbolic phase kept flags
         cudaError_t e = P->esc[b] ? launch_esc_bin(t, o, base, cnt_out, rows, vals, true, P->dtype,
-                                                   P->esc_shape_of[b], P->dev.sms, sb)
+                                                   P->dev.sms, sb)
                                   : launch_numeric_bin(t, o, base, rows, vals, P->dtype, P->num_geo[b], sb);
         if (e != cudaSuccess) return SPG_ERR_CUDA;
         if (P->timing && cudaEventRecord(P->ev1[b], sb) != cudaSuccess) return SPG_ERR_CUDA;
@@ -599,7 +598,7 @@ spg_status spgemm_numeric(spg_plan *P, const spg_csc *A, const spg_csc *B, const
         if (cudaGetLastError() != cudaSuccess) return SPG_ERR_CUDA;
     }
     Operands o{A->colptr, P->compact ? P->arow() : A->rowidx, A->values, B->colptr, B->rowidx, B->values,
-               P->compact ? P->rinv() : nullptr};
+               P->compact ? P->rinv() : nullptr, std::max(A->nnz, B->nnz)};
     return run_numeric(P, o, C_colptr, nullptr, C_rowidx, C_values, s);
 }
 
@@ -675,7 +674,7 @@ spg_status spgemm_single_pass_finish(spg_plan *P, const spg_csc *A, const spg_cs
     }
     P->num_geo_ready = true;
     Operands o{A->colptr, P->compact ? P->arow() : A->rowidx, A->values, B->colptr, B->rowidx, B->values,
-               P->compact ? P->rinv() : nullptr};
+               P->compact ? P->rinv() : nullptr, std::max(A->nnz, B->nnz)};
     st = run_numeric(P, o, soff, C_colptr, reinterpret_cast<int32_t *>(P->slots + P->srow_at), P->slots + P->sval_at, s);
     if (st != SPG_OK) return st;
     CK(P->scan_and_read(C_colptr, s));

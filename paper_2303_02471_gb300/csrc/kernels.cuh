@@ -913,6 +913,7 @@ struct Operands {
     const int64_t *Acp; const int32_t *Arow; const void *Aval;
     const int64_t *Bcp; const int32_t *Brow; const void *Bval;
     const int32_t *Rmap = nullptr;  // C's row of a compact row (numeric)
+    int64_t nnz_max = INT64_MAX;    // the larger number of entries of A and B, where known
 };
 
 // symbolic.cu
