@@ -411,32 +411,9 @@ __device__ __forceinline__ void cta_walk_bwd(const TOps<VT> &o, int64_t p0, int6
     const unsigned upto = lane == 31 ? 0xffffffffu : ((2u << lane) - 1u);
     const uint64_t pol = keep_policy();
     for (int64_t base = p0; base < p1; base += T) {
-        const int64_t p = base + threadIdx.x;
-        int z = 0;
-        int64_t a0 = 0;
-        VT bv = VT(0);
-        if (p < p1) {
-            const int32_t k = o.Brow[p];
-            a0 = o.Acp[k];
-            z = (int)(o.Acp[k + 1] - a0);
-            bv = o.Bval[p];
-        }
-        const bool lng = z >= kLongEntry;
-        // counters: long windows, long entries, short products, short entries
-        int v[4] = {lng ? (z + 31) >> 5 : 0, lng ? 1 : 0, lng ? 0 : z, (!lng && z > 0) ? 1 : 0};
-        const int mine0 = v[0], mine2 = v[2];
         int tot[4];
-        cta_incl_scan4(v, w.warp, tot);
+        walk_chunk<true, VT>(o.Acp, o.Brow, o.Bval, base, p1, w, tot, pidx);
         const int nl = tot[1];
-        if (z > 0) {
-            const int i = lng ? v[1] - 1 : nl + v[3] - 1;
-            w.key[i] = lng ? v[0] - mine0 : v[2] - mine2;
-            w.z[i] = z;
-            w.a0[i] = a0;
-            w.bv[i] = bv;
-            pidx[i] = (int32_t)threadIdx.x;
-        }
-        __syncthreads();
         const int WL = tot[0], nsh = tot[3], ZS = tot[2];
         const int64_t nwin = (int64_t)WL + ((ZS + 31) >> 5);
         const int win0 = (int)(nwin * warp / nw), win1 = (int)(nwin * (warp + 1) / nw);

@@ -212,10 +212,82 @@ __device__ __forceinline__ WalkSmem<VT> carve_walk(unsigned char *p) {
     return w;
 }
 
+// Lists the non-empty entries among B entries [base, min(base + blockDim, p1))
+// in `w`, long ones first, and returns long windows, long entries, short
+// products and short entries in tot on every thread.  At most 32 entries (most
+// columns of a sparse product) are listed by the first warp alone: the block
+// scan's barriers and seven idle warps' share of it cost more than the entries.
+// pidx (may be null): the entries' places in the chunk.  Every thread must
+// call it; a barrier must separate it from earlier readers of w.
+template <bool VALS, typename VT>
+__device__ __forceinline__ void walk_chunk(const int64_t *__restrict__ Acp, const int32_t *__restrict__ Brow,
+                                           const VT *__restrict__ Bval, int64_t base, int64_t p1,
+                                           const WalkSmem<VT> &w, int (&tot)[4], int32_t *pidx = nullptr) {
+    const int lane = threadIdx.x & 31;
+    const bool few = p1 - base <= 32;  // uniform over the CTA
+    if (!few || threadIdx.x < 32) {
+        const int64_t p = base + threadIdx.x;
+        int z = 0;
+        int64_t a0 = 0;
+        VT bv = VT(0);
+        if (p < p1) {
+            const int32_t k = Brow[p];
+            a0 = Acp[k];
+            z = (int)(Acp[k + 1] - a0);
+            if (VALS) bv = Bval[p];
+        }
+        const bool lng = z >= kLongEntry, sht = z > 0 && !lng;
+        int at, key, nl;  // the entry's place in the list and its key
+        if (few) {
+            const unsigned lm = __ballot_sync(0xffffffffu, lng), sm = __ballot_sync(0xffffffffu, sht);
+            const unsigned lt = (1u << lane) - 1u;
+            nl = __popc(lm);
+            at = lng ? __popc(lm & lt) : nl + __popc(sm & lt);
+            const int lw = lng ? (z + 31) >> 5 : 0, sp = sht ? z : 0;
+            int li = lw, si = sp;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int l = __shfl_up_sync(0xffffffffu, li, d), h = __shfl_up_sync(0xffffffffu, si, d);
+                if (lane >= d) {
+                    li += l;
+                    si += h;
+                }
+            }
+            key = lng ? li - lw : si - sp;
+            if (lane == 31) {
+                int *t = reinterpret_cast<int *>(w.warp);
+                t[0] = li;
+                t[1] = nl;
+                t[2] = si;
+                t[3] = __popc(sm);
+            }
+        } else {
+            int v[4] = {lng ? (z + 31) >> 5 : 0, lng ? 1 : 0, sht ? z : 0, sht ? 1 : 0};
+            const int m0 = v[0], m2 = v[2];
+            cta_incl_scan4(v, w.warp, tot);
+            nl = tot[1];
+            at = lng ? v[1] - 1 : nl + v[3] - 1;
+            key = lng ? v[0] - m0 : v[2] - m2;
+        }
+        if (z > 0) {
+            w.key[at] = key;
+            w.z[at] = z;
+            w.a0[at] = a0;
+            if (VALS) w.bv[at] = bv;
+            if (pidx) pidx[at] = (int32_t)threadIdx.x;
+        }
+    }
+    __syncthreads();
+    if (few) {
+        const int *t = reinterpret_cast<const int *>(w.warp);
+        for (int i = 0; i < 4; ++i) tot[i] = t[i];
+    }
+}
+
 // The whole CTA walks the products of B entries [p0, p1) of one column
-// (whose Op_j must be below 2^31).  Per chunk of blockDim entries, one block
-// scan sorts the non-empty entries into long ones (Z^A_k >= kLongEntry) and
-// short ones.  The work is cut into windows of 32 products, one per lane,
+// (whose Op_j must be below 2^31).  Per chunk of blockDim entries, walk_chunk
+// sorts the non-empty entries into long ones (Z^A_k >= kLongEntry) and short
+// ones.  The work is cut into windows of 32 products, one per lane,
 // with consecutive lanes on consecutive entries of an A column (coalesced):
 //   * a long entry contributes ceil(Z^A_k / 32) windows of its own; the
 //     window's owner is the same for all lanes and advances with a uniform
@@ -245,37 +317,9 @@ __device__ __forceinline__ void cta_walk(const int64_t *__restrict__ Acp, const 
     const unsigned upto = lane == 31 ? 0xffffffffu : ((2u << lane) - 1u);
     const uint64_t pol = keep_policy();
     for (int64_t base = p0; base < p1; base += T) {
-        const int64_t p = base + threadIdx.x;
-        int z = 0;
-        int64_t a0 = 0;
-        VT bv = VT(0);
-        if (p < p1) {
-            const int32_t k = Brow[p];
-            a0 = Acp[k];
-            z = (int)(Acp[k + 1] - a0);
-            if (VALS) bv = Bval[p];
-        }
-        const bool lng = z >= kLongEntry;
-        // counters: long windows, long entries, short products, short entries
-        int v[4] = {lng ? (z + 31) >> 5 : 0, lng ? 1 : 0, lng ? 0 : z, (!lng && z > 0) ? 1 : 0};
-        const int mine[4] = {v[0], v[1], v[2], v[3]};
         int tot[4];
-        cta_incl_scan4(v, w.warp, tot);
+        walk_chunk<VALS, VT>(Acp, Brow, Bval, base, p1, w, tot);
         const int nl = tot[1];
-        if (lng) {
-            const int i = v[1] - 1;
-            w.key[i] = v[0] - mine[0];
-            w.z[i] = z;
-            w.a0[i] = a0;
-            if (VALS) w.bv[i] = bv;
-        } else if (z > 0) {
-            const int i = nl + v[3] - 1;
-            w.key[i] = v[2] - mine[2];
-            w.z[i] = z;
-            w.a0[i] = a0;
-            if (VALS) w.bv[i] = bv;
-        }
-        __syncthreads();
         const int WL = tot[0], nsh = tot[3], ZS = tot[2];
         const int WS = (ZS + 31) >> 5;
         const int64_t nwin = (int64_t)WL + WS;
@@ -289,7 +333,50 @@ __device__ __forceinline__ void cta_walk(const int64_t *__restrict__ Acp, const 
                     const int mid = (li + hi + 1) >> 1;
                     if (w.key[mid] <= win0) li = mid; else hi = mid - 1;
                 }
-                if constexpr (UB == 1 || AHEAD > 1) {
+                if constexpr (!VALS && AHEAD > 1) {
+                    // rows only, entry by entry: only the entry's last window
+                    // can be partly filled, so the others need no bounds per
+                    // lane (a third of the flag walk's instructions; with
+                    // values, where the adds to C bound the walk and 64
+                    // registers are full, this form was 4 to 13 % slower)
+                    for (int win = win0; win < e1; ++li) {
+                        const int e_key = w.key[li], e_z = w.z[li];
+                        const int nk = li + 1 < nl ? w.key[li + 1] : 0x7fffffff;
+                        const int e_end = nk < e1 ? nk : e1;
+                        const int first = win - e_key;
+                        const int32_t *rp = Arow + w.a0[li] + (first << 5) + lane;
+                        // full windows of the run, and its rest of the last one
+                        const int end = e_end - e_key, whole = e_z >> 5;
+                        const int n = (end < whole ? end : whole) - first;
+                        const int rest = end > whole ? e_z & 31 : 0;
+                        const int32_t rr = lane < rest ? ld_keep(rp + (n << 5), pol) : 0;
+                        // the ring of AHEAD windows, as below
+                        int32_t rq[AHEAD];
+#pragma unroll
+                        for (int d = 0; d < AHEAD; ++d)
+                            if (d < n) rq[d] = ld_keep(rp + 32 * d, pol);
+                        int k = n;  // windows left
+                        for (; k >= 2 * AHEAD; k -= AHEAD) {
+                            rp += 32 * AHEAD;
+#pragma unroll
+                            for (int d = 0; d < AHEAD; ++d) {
+                                f(rq[d], VT(0));
+                                rq[d] = ld_keep(rp + 32 * d, pol);
+                            }
+                        }
+#pragma unroll 1
+                        for (; k > 0; k -= AHEAD) {
+                            rp += 32 * AHEAD;
+#pragma unroll
+                            for (int d = 0; d < AHEAD; ++d) {
+                                if (d < k) f(rq[d], VT(0));
+                                if (d + AHEAD < k) rq[d] = ld_keep(rp + 32 * d, pol);
+                            }
+                        }
+                        if (lane < rest) f(rr, VT(0));
+                        win = e_end;
+                    }
+                } else if constexpr (UB == 1 || AHEAD > 1) {
                     // entry by entry: the entry's windows in [win, e_end)
                     // are one warp-uniform loop over idx = window * 32 + lane
                     // of its A column

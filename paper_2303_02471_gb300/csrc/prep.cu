@@ -200,12 +200,16 @@ __device__ __forceinline__ int64_t mod_by(unsigned long long x, unsigned long lo
     return (int64_t)r;
 }
 
+// floor(log2(op)) of a column with products.
+__device__ __forceinline__ int op_class(int64_t op) { return op >> 31 ? 31 : 31 - __clz((int)op); }
+
 __global__ void __launch_bounds__(kCountThreads) k_count_bin(CountArgs a, Ctrl *ctrl) {
     __shared__ unsigned long long s_hist[NBINS];
     __shared__ unsigned long long s_max[NBINS];
     __shared__ unsigned long long s_binprod[NBINS];
     __shared__ unsigned long long s_binb[NBINS];
     __shared__ unsigned long long s_prod, s_cap;
+    __shared__ unsigned s_cls[32];
     __shared__ int64_t s_op[kCountThreads];    // Op of the CTA's columns
     __shared__ int s_long[kCountThreads];      // columns (thread indices) of more than kCountShort entries
     __shared__ int64_t s_lp[kCountThreads];    // their first entry
@@ -219,6 +223,7 @@ __global__ void __launch_bounds__(kCountThreads) k_count_bin(CountArgs a, Ctrl *
         s_binprod[threadIdx.x] = 0;
         s_binb[threadIdx.x] = 0;
     }
+    if (threadIdx.x < 32) s_cls[threadIdx.x] = 0;
     if (threadIdx.x == 0) s_prod = s_cap = 0;
     const RowRule rows = row_rule((int64_t)ctrl->mrows, a.mA);
     const int64_t t = effective_t(a.t, a.hmax, rows.m);
@@ -307,6 +312,7 @@ __global__ void __launch_bounds__(kCountThreads) k_count_bin(CountArgs a, Ctrl *
             cap += (unsigned long long)(s < rows.m ? s : rows.m);
             b = bin_of(s, t, a.hmax, a.promote);
             if (b == BIN_EMPTY) a.Ccp[j + 1] = 0;
+            if (b == BIN_DENSE) atomicAdd(&s_cls[op_class(s)], 1u);
         }
         // per-bin statistics, one group of lanes per bin present; sums of 32
         // values below 2^26 fit 32 bits (else 64-bit butterflies)
@@ -361,6 +367,8 @@ __global__ void __launch_bounds__(kCountThreads) k_count_bin(CountArgs a, Ctrl *
         atomicAdd(&ctrl->binprod[threadIdx.x], s_binprod[threadIdx.x]);
         atomicAdd(&ctrl->binnnzb[threadIdx.x], s_binb[threadIdx.x]);
     }
+    if (threadIdx.x < 32 && s_cls[threadIdx.x])
+        atomicAdd(&ctrl->cls[threadIdx.x], (unsigned long long)s_cls[threadIdx.x]);
     if (threadIdx.x == 0) {
         atomicAdd(&ctrl->products, s_prod);
         atomicAdd(&ctrl->capsum, s_cap);
@@ -513,70 +521,87 @@ cudaError_t launch_slot_copy(int64_t nB, int64_t nnzC, const int64_t *Ccp, const
 
 int64_t copy_tile_count(int64_t n) { return n / kCopyTile + 2; }
 
-// Column ids into per-bin lists (each block reserves its slots with one
-// global atomic per bin, so columns of a bin stay roughly in ascending order
-// within a block's tile).  The lists start at the running sums of the bins'
-// counts, taken from the control block, so nothing of it waits for the host;
-// block 0 then writes the control block to the host's mirror (the host reads
-// its counts and errors, not the scatter cursors this kernel moves).
+// Column ids into per-bin lists, the dense bin's by class (see next_dense).  A
+// block lists its columns in ascending order and reserves its slots with one
+// global atomic per list, so a list ascends within a block's tile and roughly
+// over them.  The lists start at the running sums of their counts, taken from
+// the control block, so nothing of it waits for the host; block 0 then writes
+// the control block to the host's mirror (the host reads its counts and
+// errors, not the scatter cursors this kernel moves).
 constexpr int kScatterThreads = 256;
-constexpr int kScatterItems = 4;  // columns per thread: fewer blocks on the bins' cursors
+constexpr int kScatterItems = 4;  // columns per thread: fewer blocks on the lists' cursors
+constexpr int kScatterLists = NBINS + 32;  // a bin, or NBINS + a class of the dense bin
+constexpr int kScatterParts = kScatterItems * kScatterThreads / 32;
 
 __global__ void __launch_bounds__(kScatterThreads) k_bin_scatter(const int64_t *__restrict__ op, int64_t nB,
                                                                 int64_t tcfg, int64_t hmax, int promote, int64_t mA,
                                                                 int32_t *__restrict__ bin_cols, Ctrl *ctrl,
                                                                 unsigned char *host) {
-    __shared__ unsigned int s_cnt[NBINS];
-    __shared__ unsigned long long s_base[NBINS];
+    // columns of each list in the warps' parts of the tile, then before them
+    __shared__ unsigned int s_cnt[kScatterParts][kScatterLists];
+    __shared__ unsigned long long s_base[kScatterLists];
     if (host && blockIdx.x == 0)
         for (int i = threadIdx.x; i < (int)(sizeof(Ctrl) / 8); i += kScatterThreads)
             reinterpret_cast<unsigned long long *>(host)[i] = reinterpret_cast<const unsigned long long *>(ctrl)[i];
     if (ctrl->err || !bin_cols) return;  // Op is not there for a malformed product
-    if (threadIdx.x < NBINS) s_cnt[threadIdx.x] = 0;
+    for (int i = threadIdx.x; i < kScatterParts * kScatterLists; i += kScatterThreads) (&s_cnt[0][0])[i] = 0u;
     __syncthreads();
     const int64_t t = effective_t(tcfg, hmax, row_rule((int64_t)ctrl->mrows, mA).m);
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t j0 = (int64_t)blockIdx.x * (kScatterThreads * kScatterItems) + threadIdx.x;
     int b[kScatterItems];
     unsigned r[kScatterItems];
 #pragma unroll
     for (int u = 0; u < kScatterItems; ++u) {
         const int64_t j = j0 + u * kScatterThreads;
-        b[u] = j < nB ? bin_of(op[j], t, hmax, promote) : BIN_EMPTY;
+        const int64_t o = j < nB ? op[j] : 0;
+        b[u] = bin_of(o, t, hmax, promote);
+        if (b[u] == BIN_DENSE) b[u] = NBINS + op_class(o);
         r[u] = 0;
     }
 #pragma unroll
     for (int u = 0; u < kScatterItems; ++u) {
         unsigned pending = __ballot_sync(0xffffffffu, b[u] != BIN_EMPTY);
         while (pending) {
-            const int leader = __ffs(pending) - 1;
-            const int bb = __shfl_sync(0xffffffffu, b[u], leader);
+            const int bb = __shfl_sync(0xffffffffu, b[u], __ffs(pending) - 1);
             const unsigned m = __ballot_sync(0xffffffffu, b[u] == bb);
-            unsigned at = 0;
-            if (lane == leader) at = atomicAdd(&s_cnt[bb], (unsigned)__popc(m));
-            at = __shfl_sync(0xffffffffu, at, leader);
-            if (b[u] == bb) r[u] = at + __popc(m & ((1u << lane) - 1u));
+            if (b[u] == bb) r[u] = __popc(m & ((1u << lane) - 1u));
+            if (lane == 0) s_cnt[u * (kScatterThreads / 32) + warp][bb] = __popc(m);
             pending &= ~m;
         }
     }
     __syncthreads();
-    if (threadIdx.x < NBINS && s_cnt[threadIdx.x]) {
-        unsigned long long off = 0;
-        for (int i = BIN_EMPTY + 1; i < (int)threadIdx.x; ++i) off += ctrl->hist[i];
-        s_base[threadIdx.x] = off + atomicAdd(&ctrl->fill[threadIdx.x], (unsigned long long)s_cnt[threadIdx.x]);
+    if (threadIdx.x < kScatterLists) {
+        const int l = threadIdx.x;
+        unsigned n = 0;
+        for (int p = 0; p < kScatterParts; ++p) {
+            const unsigned c = s_cnt[p][l];
+            s_cnt[p][l] = n;
+            n += c;
+        }
+        if (n) {
+            // the lists of the bins before, and of the heavier classes
+            unsigned long long off = 0;
+            for (int i = BIN_EMPTY + 1; i < (l < NBINS ? l : BIN_DENSE); ++i) off += ctrl->hist[i];
+            for (int c = 31; l >= NBINS && c > l - NBINS; --c) off += ctrl->cls[c];
+            unsigned long long *fill = l < NBINS ? &ctrl->fill[l] : &ctrl->clsfill[l - NBINS];
+            s_base[l] = off + atomicAdd(fill, (unsigned long long)n);
+        }
     }
     __syncthreads();
 #pragma unroll
     for (int u = 0; u < kScatterItems; ++u)
-        if (b[u] != BIN_EMPTY) bin_cols[(int64_t)s_base[b[u]] + r[u]] = (int32_t)(j0 + u * kScatterThreads);
+        if (b[u] != BIN_EMPTY)
+            bin_cols[s_base[b[u]] + s_cnt[u * (kScatterThreads / 32) + warp][b[u]] + r[u]] =
+                (int32_t)(j0 + u * kScatterThreads);
 }
 
 cudaError_t launch_bin_scatter(const CountArgs &a, int32_t *bin_cols, Ctrl *ctrl, unsigned char *host,
                                cudaStream_t s) {
     static_assert(sizeof(Ctrl) % 8 == 0, "the control block is copied in 8-byte words");
     const int64_t g = bin_cols ? std::max<int64_t>(1, ceil_div(a.nB, kScatterThreads * kScatterItems)) : 1;
-    k_bin_scatter<<<(unsigned)g, kScatterThreads, 0, s>>>(a.op, a.nB, a.t, a.hmax, a.promote, a.mA, bin_cols, ctrl,
-                                                          host);
+    k_bin_scatter<<<(unsigned)g, kScatterThreads, 0, s>>>(a.op, a.nB, a.t, a.hmax, a.promote, a.mA, bin_cols,
+                                                          ctrl, host);
     return cudaGetLastError();
 }
 

@@ -88,3 +88,26 @@ def test_malformed_operands_are_rejected(what):
     C, plan = ops.spgemm(dA, dB)
     plan.check()
     assert_matches_oracle(C, A, B)
+
+
+@pytest.mark.parametrize("heavy", [1, 5, 700])
+def test_dense_list_from_both_ends(heavy):
+    """Columns of every weight class in the dense bin, `heavy` of them far
+    heavier than the rest, forward and backward: each column is worked once."""
+    import torch
+    from paper_2303_02471_gb300 import ops
+    rng = np.random.default_rng(heavy)
+    A = _matrix(rng, 2000, rng.integers(0, 60, 900))
+    n = 1500
+    B = _matrix(rng, 900, np.where(np.arange(n) % max(1, n // heavy) == 3, 800, rng.integers(0, 12, n)))
+    dA, dB = upload(A), upload(B)
+    C, plan = ops.spgemm(dA, dB, ops.Config(t=1))
+    assert_matches_oracle(C, A, B)
+    dc = torch.as_tensor(rng.standard_normal(C.nnz), device="cuda")
+    got = ops.spgemm_backward(plan, dA, dB, C, dc)
+    plan.check()
+    Ch, d = C.to_host(), dc.cpu().numpy()
+    want = oracle.backward(A, B, Ch, d)
+    scale = oracle.backward(A.with_values(np.abs(A.values)), B.with_values(np.abs(B.values)), Ch, np.abs(d))
+    for g, r, s in zip(got, want, scale):  # sums of at most 2000 terms: 2.2e-13 of their size
+        assert np.all(np.abs(g.cpu().numpy() - r) <= 1e-12 * s)
