@@ -282,7 +282,7 @@ __device__ __forceinline__ bool num_dense_column(const TOps<VT> &o, int32_t j, i
                                                  unsigned *s_next, int32_t *Crow, VT *Cval, AP &&after_prefix,
                                                  int64_t *cnt_out = nullptr) {
     // the previous user of *s_next finished before the caller's last barrier
-    if (threadIdx.x == 0) *s_next = (blockDim.x >> 5) * kVisitGroup;
+    if (threadIdx.x == 0) *s_next = (blockDim.x >> 5) * visit_group(W);
     // flags kept from the symbolic phase are read straight into the prefix
     // pass; otherwise the walk sets them again
     if (!keep)
@@ -308,8 +308,8 @@ __device__ __forceinline__ bool num_dense_column(const TOps<VT> &o, int32_t j, i
     int32_t *crow = Crow + c0;
     // the extraction stages rows in the walk's scratch, free once cta_walk
     // has returned (it ends with a barrier): 20 bytes per thread
-    static_assert(kVisitStage * 4 <= 32 * (16 + sizeof(float)), "visit staging exceeds the walk scratch");
-    int32_t *stage = reinterpret_cast<int32_t *>(w.a0);
+    static_assert(kVisitBytes <= 32 * (16 + sizeof(float)), "visit staging exceeds the walk scratch");
+    unsigned char *stage = reinterpret_cast<unsigned char *>(w.a0);
     for (int32_t i = threadIdx.x; i < n32; i += blockDim.x) gacc[i] = VT(0);
     __syncthreads();
     cta_walk<true, VT, kWalkAhead>(o.Acp, o.Arow, o.Aval, o.Brow, o.Bval, o.Bcp[j], o.Bcp[j + 1], w,

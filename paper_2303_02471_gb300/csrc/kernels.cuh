@@ -728,34 +728,47 @@ __device__ __forceinline__ int64_t cta_bitmap_prefix(uint2 *bm, int64_t W64, con
 
 // Writes out the set bits of bm[0..W) in ascending row order: the row at
 // sorted position `rank` of the column is stored by put(rank, map(row))
-// (bm[..].y must hold the prefix counts).  Warps take groups of kVisitGroup
-// chunks of 32 words, the first group by warp index and the next ones from
-// the shared counter *s_next, which must hold kVisitGroup * (number of warps)
-// before a barrier that precedes the call (one shared atomic per 4096 rows).
-// The ranks of a group are consecutive: each lane holds one word of a chunk
-// and writes the word's rows, rank minus the group's first rank being the
-// slot, into the warp's kVisitStage-entry slice of `stage`; the warp then
-// stores the staged slots in order, one per lane, with kVisitUnroll map()
-// look-ups in flight per lane before their stores, so the stores are
-// coalesced and a group waits for few look-up latencies.  A group of more
-// than kVisitStage rows goes through the slice in pieces.  stage:
-// kVisitStage ints per warp of shared memory that nothing else uses during
-// the call.  Clears the bits when `clear`.  No barrier inside.
-// Chunks of 32 words a warp takes per grab in cta_bitmap_visit.
+// (bm[..].y must hold the prefix counts).  Warps take groups of
+// visit_group(W) chunks of 32 words, the first group by warp index and the
+// next ones from the shared counter *s_next, which must hold
+// visit_group(W) * (number of warps) before a barrier that precedes the call.
+// A warp first lists the group's non-empty words (two thirds of the words of a
+// power-law product's columns are empty), then takes 32 of them at a time, one
+// per lane (R-MAT 2^16 in float 1158 -> 1132 us, R-MAT 2^17's numeric phase
+// 2018 -> 1995 us: the pass was over half of the kernel's instructions, but
+// the adds of the walk bound it).  The ranks of a group are consecutive: a lane writes its word's
+// rows, rank minus the group's first rank being the slot, into the warp's
+// slice of shared memory; the warp then stores the staged slots in order, one
+// per lane, with kVisitUnroll map() look-ups in flight per lane before their
+// stores, so the stores are coalesced and a group waits for few look-up
+// latencies.  A group of more than kVisitStage rows goes through the slice in
+// pieces.  stage: kVisitBytes per warp of shared memory that nothing else uses
+// during the call.  Clears the bits when `clear`.  No barrier inside.
+// Most chunks of 32 words a warp takes per grab (fewer where the warps would
+// otherwise run out of groups).
 constexpr int kVisitGroup = 4;
-// Rows a warp stages per piece in cta_bitmap_visit.
-constexpr int kVisitStage = 160;
-// Look-ups per lane issued before their stores in cta_bitmap_visit.
+// Rows a warp stages per piece.
+constexpr int kVisitStage = 128;
+// Look-ups per lane issued before their stores.
 constexpr int kVisitUnroll = 4;
+// Staged rows and the list of words (offsets in the group).
+constexpr int kVisitBytes = kVisitStage * 4 + kVisitGroup * 32;
+
+__device__ __forceinline__ int visit_group(int64_t W) {
+    const int per = ((int)((W + 31) >> 5) * 32) / (int)blockDim.x;  // chunks per warp
+    return per >= kVisitGroup ? kVisitGroup : per < 1 ? 1 : per;
+}
 
 template <typename M, typename P>
 __device__ __forceinline__ void cta_bitmap_visit(uint2 *bm, int64_t W64, bool clear, unsigned *s_next,
-                                                 int32_t *stage, M &&map, P &&put) {
+                                                 unsigned char *stage, M &&map, P &&put) {
     // m < 2^31, so words, chunks and ranks all fit 32-bit indices
     const int W = (int)W64;
     const int lane = threadIdx.x & 31;
-    const int nchunks = (W + 31) >> 5;
-    int32_t *slots = stage + (threadIdx.x >> 5) * kVisitStage;
+    const int nchunks = (W + 31) >> 5, group = visit_group(W64);
+    int32_t *slots = reinterpret_cast<int32_t *>(stage + (threadIdx.x >> 5) * kVisitBytes);
+    unsigned char *words = reinterpret_cast<unsigned char *>(slots + kVisitStage);
+    const unsigned lt = (1u << lane) - 1u;
     // stores the slots of relative ranks [from, to), slot 0 holding `from`
     auto flush = [&](int32_t r0, int from, int to) {
         for (int o0 = from; o0 < to; o0 += 32 * kVisitUnroll) {
@@ -772,43 +785,66 @@ __device__ __forceinline__ void cta_bitmap_visit(uint2 *bm, int64_t W64, bool cl
             }
         }
     };
-    for (int g = (threadIdx.x >> 5) * kVisitGroup; g < nchunks;) {
-        const int gend = g + kVisitGroup < nchunks ? g + kVisitGroup : nchunks;
-        // the group's first word exists (g < nchunks); its prefix count is
-        // the group's first rank
-        const int32_t r0 = (int32_t)bm[g << 5].y;
-        int flushed = 0;  // relative ranks below this are stored
-        int top = 0;      // relative end of the rows staged so far
+    for (int g = (threadIdx.x >> 5) * group; g < nchunks;) {
+        const int gend = g + group < nchunks ? g + group : nchunks;
+        const int w0 = g << 5;
+        int n = 0;  // non-empty words
         for (int c = g; c < gend; ++c) {
             const int wd = (c << 5) + lane;
-            const uint2 v = wd < W ? bm[wd] : make_uint2(0u, 0u);
-            if (clear && v.x) bm[wd].x = 0u;
-            uint32_t bits = v.x;
-            // lanes past W hold no bits
-            int pos = wd < W ? (int)v.y - r0 : 0;
-            const int32_t row0 = wd << 5;
-            const int end = (int)__reduce_max_sync(0xffffffffu, (unsigned)(pos + __popc(bits)));
-            for (;;) {
-                const int lim = flushed + kVisitStage;
-                while (bits && pos < lim) {
-                    const int b = __ffs(bits) - 1;
-                    bits &= bits - 1u;
-                    slots[pos - flushed] = row0 + b;
-                    ++pos;
-                }
-                if (end <= lim) break;  // uniform over the warp
-                __syncwarp();
-                flush(r0, flushed, lim);
-                __syncwarp();
-                flushed = lim;
+            const bool set = wd < W && bm[wd].x != 0u;
+            const unsigned m = __ballot_sync(0xffffffffu, set);
+            if (set) words[n + __popc(m & lt)] = (unsigned char)(wd - w0);
+            n += __popc(m);
+        }
+        __syncwarp();
+        // the group's first word exists (g < nchunks); its prefix count is
+        // the group's first rank
+        const int32_t r0 = (int32_t)bm[w0].y;
+        int flushed = 0;  // relative ranks below this are stored
+        int top = 0;      // relative end of the rows staged so far
+        for (int i0 = 0; i0 < n; i0 += 32) {
+            const int i = i0 + lane;
+            uint32_t bits = 0u;
+            int pos = 0;
+            int32_t row0 = 0;
+            if (i < n) {
+                const int wd = w0 + words[i];
+                const uint2 v = bm[wd];
+                if (clear) bm[wd].x = 0u;
+                bits = v.x;
+                pos = (int)v.y - r0;
+                row0 = wd << 5;
             }
-            top = end > top ? end : top;
+            const int end = (int)__reduce_max_sync(0xffffffffu, (unsigned)(pos + __popc(bits)));
+            // whole in the slice (uniform over the warp), else in pieces
+            if (end <= flushed + kVisitStage) {
+                int32_t *to = slots + (pos - flushed);
+                while (bits) {
+                    *to++ = row0 + __ffs(bits) - 1;
+                    bits &= bits - 1u;
+                }
+            } else {
+                for (;;) {
+                    const int lim = flushed + kVisitStage;
+                    while (bits && pos < lim) {
+                        slots[pos - flushed] = row0 + __ffs(bits) - 1;
+                        bits &= bits - 1u;
+                        ++pos;
+                    }
+                    if (end <= lim) break;  // uniform over the warp
+                    __syncwarp();
+                    flush(r0, flushed, lim);
+                    __syncwarp();
+                    flushed = lim;
+                }
+            }
+            top = end;
         }
         __syncwarp();
         flush(r0, flushed, top);
         __syncwarp();
         unsigned nc = 0;
-        if (lane == 0) nc = atomicAdd(s_next, (unsigned)kVisitGroup);
+        if (lane == 0) nc = atomicAdd(s_next, (unsigned)group);
         g = (int)__shfl_sync(0xffffffffu, nc, 0);
     }
 }
