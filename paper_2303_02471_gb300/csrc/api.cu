@@ -190,6 +190,12 @@ struct spg_plan {
         host = got.ctrl;
         return cudaSuccess;
     }
+    // the dynamic work counters to zero, where a bin of the plan uses one
+    bool reset_work(cudaStream_t s) const {
+        bool used = false;
+        for (int b = BIN_CTA0; b < NBINS; ++b) used |= host.hist[b] != 0;
+        return !used || cudaMemsetAsync(&ctrl()->work, 0, sizeof(Ctrl::work), s) == cudaSuccess;
+    }
     int64_t nonempty_bins() const {
         int64_t n = 0;
         for (int b = 1; b < NBINS; ++b) n += host.hist[b] ? 1 : 0;
@@ -589,7 +595,7 @@ spg_status spgemm_numeric(spg_plan *P, const spg_csc *A, const spg_csc *B, const
     if (!C_colptr || (P->nnzC > 0 && (!C_rowidx || !C_values))) return SPG_ERR_INVALID;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     Ctrl *ctrl = P->ctrl();
-    if (cudaMemsetAsync(&ctrl->work, 0, sizeof(ctrl->work), s) != cudaSuccess) return SPG_ERR_CUDA;
+    if (!P->reset_work(s)) return SPG_ERR_CUDA;
     if (P->compact && P->nnzA > 0) {
         // A's rows renumbered again from the A given here: an entry in a row
         // that held none at planning time is reported, not walked
@@ -734,7 +740,7 @@ spg_status spgemm_backward(spg_plan *P, const spg_csc *A, const spg_csc *B, cons
         return SPG_ERR_CUDA;
     if (!dA_values && !dB_values) return SPG_OK;
     Ctrl *ctrl = P->ctrl();
-    if (cudaMemsetAsync(&ctrl->work, 0, sizeof(ctrl->work), s) != cudaSuccess) return SPG_ERR_CUDA;
+    if (!P->reset_work(s)) return SPG_ERR_CUDA;
     if (!P->bwd_geo_ready) {
         for (int b = 1; b < NBINS; ++b) {
             if (!P->host.hist[b]) continue;

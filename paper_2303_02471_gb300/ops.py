@@ -118,8 +118,7 @@ class Config:
     group_promote: Optional[int] = None      # lane-group bins a light column moves up (0..2)
 
     def native(self) -> N.SpgConfig:
-        c = N.SpgConfig()
-        N.check(N.lib().spg_config_default(ctypes.byref(c)), "spg_config_default")
+        c = _default_config()
         for f in ("t", "hash_cta_max", "cta_threads", "table_shrink", "scratch_cap_bytes",
                   "dense_cache_bytes", "table_slots_pct", "group_promote"):
             v = getattr(self, f)
@@ -136,6 +135,16 @@ class Config:
 
 
 _DT = {torch.float64: N.SPG_F64, torch.float32: N.SPG_F32}
+_DEFAULTS = []
+
+
+def _default_config() -> N.SpgConfig:
+    """A copy of the library's default configuration (asked for once)."""
+    if not _DEFAULTS:
+        c = N.SpgConfig()
+        N.check(N.lib().spg_config_default(ctypes.byref(c)), "spg_config_default")
+        _DEFAULTS.append(bytes(c))
+    return N.SpgConfig.from_buffer_copy(_DEFAULTS[0])
 
 
 def _ptr(t: Optional[torch.Tensor]):
@@ -143,19 +152,26 @@ def _ptr(t: Optional[torch.Tensor]):
 
 
 def _csc(M: CscMatrix, dtype=None) -> N.SpgCsc:
-    dt = dtype if dtype is not None else M.dtype
-    if dt not in _DT:
+    cp, ri, v = M.colptr, M.rowidx, M.values
+    dt = dtype if dtype is not None else v.dtype if v is not None else torch.float64
+    code = _DT.get(dt)
+    if code is None:
         raise TypeError(f"unsupported dtype {dt}")
-    for t, want in ((M.colptr, torch.int64), (M.rowidx, torch.int32)):
-        if t.dtype != want or not t.is_contiguous() or not t.is_cuda:
-            raise TypeError("CSC index arrays must be contiguous CUDA int64 colptr / int32 rowidx")
-    if M.values is not None and (not M.values.is_contiguous() or not M.values.is_cuda):
+    if not (cp.dtype is torch.int64 and ri.dtype is torch.int32 and cp.is_cuda and ri.is_cuda and
+            cp.is_contiguous() and ri.is_contiguous()):
+        raise TypeError("CSC index arrays must be contiguous CUDA int64 colptr / int32 rowidx")
+    if v is not None and not (v.is_cuda and v.is_contiguous()):
         raise TypeError("CSC values must be a contiguous CUDA tensor")
-    return N.SpgCsc(M.nrows, M.ncols, M.nnz, M.colptr.data_ptr(), _ptr(M.rowidx),
-                    _ptr(M.values), _DT[dt])
+    return N.SpgCsc(M.nrows, M.ncols, ri.shape[0], cp.data_ptr(), ri.data_ptr() if ri.numel() else None,
+                    v.data_ptr() if v is not None and v.numel() else None, code)
+
+
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(stream=None):
+    if stream is None and _raw_stream is not None:  # without a Stream object
+        return ctypes.c_void_p(_raw_stream(torch.cuda.current_device()))
     s = stream if stream is not None else torch.cuda.current_stream()
     return ctypes.c_void_p(s.cuda_stream)
 
@@ -284,24 +300,20 @@ class Plan:
             pass
 
 
-def workspace_size(A: CscMatrix, B: CscMatrix, config: Optional[Config] = None) -> int:
-    cfg = (config or Config()).native()
+def _workspace_size(cA, cB, cfg) -> int:
     nbytes = ctypes.c_size_t()
-    N.check(N.lib().spgemm_workspace_size(ctypes.byref(_csc(A)), ctypes.byref(_csc(B, A.dtype)),
-                                          ctypes.byref(cfg), ctypes.byref(nbytes)),
-            "spgemm_workspace_size")
+    N.check(N.lib().spgemm_workspace_size(ctypes.byref(cA), ctypes.byref(cB), ctypes.byref(cfg),
+                                          ctypes.byref(nbytes)), "spgemm_workspace_size")
     return nbytes.value
 
 
-def spgemm_symbolic(A: CscMatrix, B: CscMatrix, config: Optional[Config] = None,
-                    workspace: Optional[torch.Tensor] = None, lib_handle: Optional[Handle] = None):
-    """Column pointers of C = A B, nnz(C) and the plan (synchronises).
-    lib_handle: the Handle to use (default: the device's shared one)."""
-    config = config or Config()
-    hd = lib_handle if lib_handle is not None else handle(A.device)
+def workspace_size(A: CscMatrix, B: CscMatrix, config: Optional[Config] = None) -> int:
+    return _workspace_size(_csc(A), _csc(B, A.dtype), (config or Config()).native())
+
+
+def _symbolic(A, B, cA, cB, config, workspace, hd):
     cfg = config.native()
-    cA, cB = _csc(A), _csc(B, A.dtype)
-    need = workspace_size(A, B, config)
+    need = _workspace_size(cA, cB, cfg)
     if workspace is None or workspace.numel() < need:
         workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=A.device)
     colptr = torch.empty(B.ncols + 1, dtype=torch.int64, device=A.device)
@@ -314,24 +326,36 @@ def spgemm_symbolic(A: CscMatrix, B: CscMatrix, config: Optional[Config] = None,
     return colptr, nnz.value, Plan(h, workspace, A, B, colptr, nnz.value, config, hd)
 
 
-def spgemm_numeric(plan: Plan, A: CscMatrix, B: CscMatrix, rowidx: Optional[torch.Tensor] = None,
-                   values: Optional[torch.Tensor] = None) -> CscMatrix:
-    """Rows (ascending) and values of C = A B into new or given buffers."""
+def _numeric(plan, A, B, cA, cB, rowidx, values):
     if rowidx is None:
         rowidx = torch.empty(plan.nnz, dtype=torch.int32, device=A.device)
     if values is None:
         values = torch.empty(plan.nnz, dtype=A.dtype, device=A.device)
-    N.check(N.lib().spgemm_numeric(plan.handle, ctypes.byref(_csc(A)), ctypes.byref(_csc(B)),
+    N.check(N.lib().spgemm_numeric(plan.handle, ctypes.byref(cA), ctypes.byref(cB),
                                    _ptr(plan.colptr), _ptr(rowidx), _ptr(values), _stream()),
             "spgemm_numeric")
     return CscMatrix(A.nrows, B.ncols, plan.colptr, rowidx, values)
 
 
+def spgemm_symbolic(A: CscMatrix, B: CscMatrix, config: Optional[Config] = None,
+                    workspace: Optional[torch.Tensor] = None, lib_handle: Optional[Handle] = None):
+    """Column pointers of C = A B, nnz(C) and the plan (synchronises).
+    lib_handle: the Handle to use (default: the device's shared one)."""
+    hd = lib_handle if lib_handle is not None else handle(A.device)
+    return _symbolic(A, B, _csc(A), _csc(B, A.dtype), config or Config(), workspace, hd)
+
+
+def spgemm_numeric(plan: Plan, A: CscMatrix, B: CscMatrix, rowidx: Optional[torch.Tensor] = None,
+                   values: Optional[torch.Tensor] = None) -> CscMatrix:
+    """Rows (ascending) and values of C = A B into new or given buffers."""
+    return _numeric(plan, A, B, _csc(A), _csc(B), rowidx, values)
+
+
 def spgemm(A: CscMatrix, B: CscMatrix, config: Optional[Config] = None):
     """C = A B (both phases).  Returns (C, plan)."""
-    _, _, plan = spgemm_symbolic(A, B, config)
-    C = spgemm_numeric(plan, A, B)
-    return C, plan
+    cA = _csc(A)
+    _, _, plan = _symbolic(A, B, cA, _csc(B, A.dtype), config or Config(), None, handle(A.device))
+    return _numeric(plan, A, B, cA, _csc(B), None, None), plan
 
 
 def single_pass_workspace_size(A: CscMatrix, B: CscMatrix, config: Optional[Config] = None,
@@ -513,14 +537,9 @@ def _csc_array(Ms):
     return arr
 
 
-def spgemm_batched_symbolic(As, Bs, config: Optional[Config] = None) -> BatchedPlan:
-    """Column pointers and nnz of every C_i = A_i B_i (synchronises)."""
-    if len(As) != len(Bs):
-        raise ValueError("A and B lists differ in length")
-    config = config or Config()
+def _batched_symbolic(As, Bs, cA, cB, config) -> BatchedPlan:
     cfg = config.native()
     nb = len(As)
-    cA, cB = _csc_array(As), _csc_array(Bs)
     nbytes = ctypes.c_size_t()
     N.check(N.lib().spgemm_batched_workspace_size(nb, cA, cB, ctypes.byref(cfg), ctypes.byref(nbytes)),
             "spgemm_batched_workspace_size")
@@ -541,25 +560,43 @@ def spgemm_batched_symbolic(As, Bs, config: Optional[Config] = None) -> BatchedP
     return BatchedPlan(h, ws, colptr, list(nnz[:nb]), segs, shapes, config, hd)
 
 
-def spgemm_batched_numeric(plan: BatchedPlan, As, Bs, use_graph: bool = False):
-    """All C_i in one persistent launch (optionally a replayed CUDA graph).
-    Output buffers are allocated on the first call and reused, so a captured
-    graph stays valid across calls."""
+def _batch_arrays(As, Bs):
+    if len(As) != len(Bs):
+        raise ValueError("A and B lists differ in length")
+    return _csc_array(As), _csc_array(Bs)
+
+
+def spgemm_batched_symbolic(As, Bs, config: Optional[Config] = None) -> BatchedPlan:
+    """Column pointers and nnz of every C_i = A_i B_i (synchronises)."""
+    return _batched_symbolic(As, Bs, *_batch_arrays(As, Bs), config or Config())
+
+
+def _batched_numeric(plan, As, Bs, cA, cB, use_graph):
     nb = len(As)
     if plan.outputs is None:
         plan.outputs = [(torch.empty(n, dtype=torch.int32, device=A.device),
                          torch.empty(n, dtype=A.dtype, device=A.device)) for n, A in zip(plan.nnz, As)]
     rows = (ctypes.c_void_p * max(1, nb))(*[r.data_ptr() if r.numel() else None for r, _ in plan.outputs])
     vals = (ctypes.c_void_p * max(1, nb))(*[v.data_ptr() if v.numel() else None for _, v in plan.outputs])
-    N.check(N.lib().spgemm_batched_numeric(plan.handle, _csc_array(As), _csc_array(Bs), _ptr(plan.colptr), rows,
+    N.check(N.lib().spgemm_batched_numeric(plan.handle, cA, cB, _ptr(plan.colptr), rows,
                                            vals, int(bool(use_graph)), _stream()), "spgemm_batched_numeric")
     return [CscMatrix(A.nrows, B.ncols, plan.colptr_of(i), r, v)
             for i, (A, B, (r, v)) in enumerate(zip(As, Bs, plan.outputs))]
 
 
+def spgemm_batched_numeric(plan: BatchedPlan, As, Bs, use_graph: bool = False):
+    """All C_i in one persistent launch (optionally a replayed CUDA graph).
+    Output buffers are allocated on the first call and reused, so a captured
+    graph stays valid across calls."""
+    return _batched_numeric(plan, As, Bs, _csc_array(As), _csc_array(Bs), use_graph)
+
+
 def spgemm_batched(As, Bs, config: Optional[Config] = None, use_graph: bool = False):
-    plan = spgemm_batched_symbolic(As, Bs, config)
-    return spgemm_batched_numeric(plan, As, Bs, use_graph), plan
+    # the operands' descriptions are made once, before the first phase: the
+    # GPU waits for the host between the phases
+    cA, cB = _batch_arrays(As, Bs)
+    plan = _batched_symbolic(As, Bs, cA, cB, config or Config())
+    return _batched_numeric(plan, As, Bs, cA, cB, use_graph), plan
 
 
 def spgemm_batched_backward(plan: BatchedPlan, As, Bs, Cs, dCs, need_dA: bool = True, need_dB: bool = True):
