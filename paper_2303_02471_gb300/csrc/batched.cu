@@ -101,25 +101,60 @@ __global__ void k_bcount(BTask b, int64_t ntot, int64_t *op) {
     __shared__ unsigned long long s_hist[NBINS], s_max[NBINS], s_prod[NBINS], s_nb[NBINS];
     if (threadIdx.x < NBINS) s_hist[threadIdx.x] = s_max[threadIdx.x] = s_prod[threadIdx.x] = s_nb[threadIdx.x] = 0;
     __syncthreads();
+    // a warp's columns step together, so that their statistics are summed over
+    // the warp before one shared atomic per bin present; kGather entries'
+    // chains of loads in flight per lane
+    constexpr int kGather = 4;
+    const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < ntot; g += stride) {
-        const int p = find_prob(b.col0s, b.nb, g);
-        const BProb &P = b.prob[p];
-        const int64_t j = g - P.col0;
-        const int64_t p0 = P.Bcp[j], p1 = P.Bcp[j + 1];
-        int64_t s = 0;
-        for (int64_t q = p0; q < p1; ++q) {
-            const int32_t k = P.Brow[q];
-            s += P.Acp[k + 1] - P.Acp[k];
+    for (int64_t g0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); g0 < ntot; g0 += stride) {
+        const int64_t g = g0 + lane;
+        const bool on = g < ntot;
+        int64_t s = 0, nb = 0;
+        int bin = -1;
+        if (on) {
+            const BProb &P = b.prob[find_prob(b.col0s, b.nb, g)];
+            const int64_t j = g - P.col0;
+            const int64_t p0 = P.Bcp[j], p1 = P.Bcp[j + 1];
+            nb = p1 - p0;
+            for (int64_t q = p0; q < p1; q += kGather) {
+                int32_t k[kGather];
+#pragma unroll
+                for (int u = 0; u < kGather; ++u) k[u] = q + u < p1 ? P.Brow[q + u] : -1;
+#pragma unroll
+                for (int u = 0; u < kGather; ++u)
+                    if (k[u] >= 0) s += P.Acp[k[u] + 1] - P.Acp[k[u]];
+            }
+            op[g] = s;
+            bin = bin_of(s, P.t, b.hmax, b.promote);
+            if (bin == BIN_EMPTY) P.Ccp[j + 1] = 0;
+            if (j == 0) P.Ccp[0] = 0;
         }
-        op[g] = s;
-        const int bin = bin_of(s, P.t, b.hmax, b.promote);
-        atomicAdd(&s_hist[bin], 1ULL);
-        atomicMax(&s_max[bin], (unsigned long long)s);
-        if (s) atomicAdd(&s_prod[bin], (unsigned long long)s);
-        if (p1 > p0) atomicAdd(&s_nb[bin], (unsigned long long)(p1 - p0));
-        if (bin == BIN_EMPTY) P.Ccp[j + 1] = 0;
-        if (j == 0) P.Ccp[0] = 0;
+        // sums of 32 values below 2^26 fit 32 bits (else each lane adds its own)
+        const bool small = __all_sync(0xffffffffu, s < (1 << 26) && nb < (1 << 26));
+        unsigned pending = __ballot_sync(0xffffffffu, on);
+        while (pending) {
+            const int leader = __ffs(pending) - 1;
+            const int bb = __shfl_sync(0xffffffffu, bin, leader);
+            const unsigned m = __ballot_sync(0xffffffffu, on && bin == bb);
+            const bool in = (m >> lane) & 1u;
+            if (small) {
+                const unsigned sm = __reduce_add_sync(0xffffffffu, in ? (unsigned)s : 0u);
+                const unsigned mx = __reduce_max_sync(0xffffffffu, in ? (unsigned)s : 0u);
+                const unsigned ns = __reduce_add_sync(0xffffffffu, in ? (unsigned)nb : 0u);
+                if (lane == leader) {
+                    atomicMax(&s_max[bb], (unsigned long long)mx);
+                    if (sm) atomicAdd(&s_prod[bb], (unsigned long long)sm);
+                    if (ns) atomicAdd(&s_nb[bb], (unsigned long long)ns);
+                }
+            } else if (in) {
+                atomicMax(&s_max[bb], (unsigned long long)s);
+                if (s) atomicAdd(&s_prod[bb], (unsigned long long)s);
+                if (nb) atomicAdd(&s_nb[bb], (unsigned long long)nb);
+            }
+            if (lane == leader) atomicAdd(&s_hist[bb], (unsigned long long)__popc(m));
+            pending &= ~m;
+        }
     }
     __syncthreads();
     if (threadIdx.x < NBINS && s_hist[threadIdx.x]) {
@@ -180,9 +215,12 @@ __global__ void k_bvalidate(const VMat *mats, int nm, const int64_t *col0s, int6
         const int64_t c = M.cp[j], c1 = M.cp[j + 1];
         bool bad = c1 < c || c < 0 || c1 > M.nnz || (j == 0 && c != 0) || (j == M.ncols - 1 && c1 != M.nnz);
         if (!bad)
-            for (int64_t e = c; e < c1; ++e) {
-                const int32_t r = M.row[e];
-                if (r < 0 || (int64_t)r >= M.nrows) { bad = true; break; }
+            for (int64_t e = c; e < c1; e += 4) {  // four loads in flight
+                int32_t r[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) r[u] = e + u < c1 ? M.row[e + u] : 0;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) bad |= e + u < c1 && (r[u] < 0 || (int64_t)r[u] >= M.nrows);
             }
         if (bad) set_error(ctrl, SPG_ERR_INVALID, which, g);
     }
