@@ -196,6 +196,9 @@ struct spg_plan {
         for (int b = BIN_CTA0; b < NBINS; ++b) used |= host.hist[b] != 0;
         return !used || cudaMemsetAsync(&ctrl()->work, 0, sizeof(Ctrl::work), s) == cudaSuccess;
     }
+    // the larger number of entries of A and B, where the column pointers are
+    // known to stay within it (without validation they may point anywhere)
+    int64_t entries() const { return cfg.validate ? std::max(nnzA, nnzB) : INT64_MAX; }
     int64_t nonempty_bins() const {
         int64_t n = 0;
         for (int b = 1; b < NBINS; ++b) n += host.hist[b] ? 1 : 0;
@@ -464,7 +467,7 @@ spg_status spgemm_symbolic(spg_handle *handle, const spg_csc *A, const spg_csc *
     } while (0)
 
     Operands o{A->colptr, P->compact ? P->arow() : A->rowidx, nullptr, B->colptr, B->rowidx, nullptr, nullptr,
-               std::max(A->nnz, B->nnz)};
+               P->entries()};
     // as in the numeric phase: beside a dense bin, the lane-group bins (shared
     // memory only) run on the side streams, launched after the dense kernel
     bool groups = false;
@@ -604,7 +607,7 @@ spg_status spgemm_numeric(spg_plan *P, const spg_csc *A, const spg_csc *B, const
         if (cudaGetLastError() != cudaSuccess) return SPG_ERR_CUDA;
     }
     Operands o{A->colptr, P->compact ? P->arow() : A->rowidx, A->values, B->colptr, B->rowidx, B->values,
-               P->compact ? P->rinv() : nullptr, std::max(A->nnz, B->nnz)};
+               P->compact ? P->rinv() : nullptr, P->entries()};
     return run_numeric(P, o, C_colptr, nullptr, C_rowidx, C_values, s);
 }
 
@@ -680,7 +683,7 @@ spg_status spgemm_single_pass_finish(spg_plan *P, const spg_csc *A, const spg_cs
     }
     P->num_geo_ready = true;
     Operands o{A->colptr, P->compact ? P->arow() : A->rowidx, A->values, B->colptr, B->rowidx, B->values,
-               P->compact ? P->rinv() : nullptr, std::max(A->nnz, B->nnz)};
+               P->compact ? P->rinv() : nullptr, P->entries()};
     st = run_numeric(P, o, soff, C_colptr, reinterpret_cast<int32_t *>(P->slots + P->srow_at), P->slots + P->sval_at, s);
     if (st != SPG_OK) return st;
     CK(P->scan_and_read(C_colptr, s));

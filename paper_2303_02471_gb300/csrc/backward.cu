@@ -142,8 +142,10 @@ static Geo backward_geometry_t(int bin, int64_t count, int64_t m, int threads, i
     // Dense: as in the numeric phase, several CTAs per SM overlap one
     // another's per-column barriers (backward of R-MAT 2^16 squared in
     // double: 3.07 ms with one 1024-thread CTA per SM and a segmented scan
-    // per window, 1.51 ms now): 256 threads where that
-    // keeps as many threads resident as 512, else 512.  The CTA's share of
+    // per window, 1.23 ms now): 256 threads where that
+    // keeps as many threads resident as 512, else 512; where the flags live in
+    // the per-CTA scratch, the configured size (2^20 rows: double 0.67 ms with
+    // 1024 threads, 1.09 with two CTAs of 512).  The CTA's share of
     // the SM's shared memory then holds dC[:, j] of the columns it fits.
     const size_t bmb = (size_t)W * 8;
     auto shape = [&](int tt, Geo &o) {
@@ -152,15 +154,13 @@ static Geo backward_geometry_t(int bin, int64_t count, int64_t m, int threads, i
         const size_t fx = walk_smem_bytes<VT>(tt) + al16((size_t)tt * 4);
         o.bm_global = bmb > kBitmapSmemMax || fx + bmb > smem_optin;
         o.smem = fx + (o.bm_global ? 0 : bmb);
-        int occ = occupancy(k_bwd_dense<VT, true>, tt, o.smem);
-        // flags in the per-CTA scratch: no more CTAs than it has slots for
-        if (o.bm_global) occ = (int)std::max<int64_t>(1, std::min<int64_t>(occ, scratch_ctas / sms));
-        return occ;
+        return occupancy(k_bwd_dense<VT, true>, tt, o.smem);
     };
     int occ = 0;
-    if (threads >= 512) {
-        Geo g256, g512;
-        const int o256 = shape(256, g256), o512 = shape(512, g512);
+    Geo g256, g512;
+    const int o256 = threads >= 512 ? shape(256, g256) : 0;
+    if (o256 > 0 && !g256.bm_global) {
+        const int o512 = shape(512, g512);
         if (o256 * 256 >= o512 * 512) { g = g256; occ = o256; }
         else { g = g512; occ = o512; }
     } else {
