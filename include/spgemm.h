@@ -119,16 +119,14 @@ typedef struct {
     int32_t test_wait_timeout;
     /* Accumulator of the lane-group bins (columns with Op_j <= 256):
      * SPG_ACC_HASH, the hash tables of Section 3.2, in both phases;
-     * SPG_ACC_ESC, the ESC algorithm of Section 4 (the products of a tile of
-     * columns are expanded into shared memory, sorted by (column, row) and
-     * compressed), in both phases; SPG_ACC_AUTO (default), ESC for the
-     * numeric phase and, for the symbolic phase's counts, ESC in the bins of
-     * Op_j <= 64 (sorted by rank) and hash tables in the larger ones (the
-     * cheaper in each case, measured on GB300).  A bin whose (column, row)
-     * keys do not fit 32 bits keeps hash tables.  All give the
-     * same C (the ESC sums do not depend on timing).  The single pass uses
-     * ESC unless SPG_ACC_HASH.  Only the single products use it; the batched
-     * calls keep hash tables. */
+     * SPG_ACC_ESC, the ESC algorithm of Section 4 (a column's products are
+     * expanded into a lane group's registers, sorted by row and compressed),
+     * in both phases; SPG_ACC_AUTO (default), ESC for the numeric phase and,
+     * for the symbolic phase's counts, ESC in the bins of Op_j <= 64 and hash
+     * tables in the larger ones (the cheaper in each case, measured on
+     * GB300).  All give the same C (the ESC sums do not depend on timing).
+     * The single pass uses ESC unless SPG_ACC_HASH.  Only the single products
+     * use it; the batched calls keep hash tables. */
     int32_t small_accumulator;
     /* Size of the hash tables of the numeric and backward phases' CTA and
      * global bins (Section 3.2's table size), in slots per output entry of
