@@ -215,8 +215,10 @@ __global__ void __launch_bounds__(kCountThreads) k_count_bin(CountArgs a, Ctrl *
     __shared__ int64_t s_lp[kCountThreads];    // their first entry
     __shared__ int32_t s_ln[kCountThreads];    // and number of entries
     __shared__ int s_nlong;
-    // what the row pass found: nothing here follows a malformed A
-    if (ctrl->err) return;
+    // what the row pass found: nothing here follows a malformed A.  Other CTAs
+    // of this kernel report a malformed B in the same word meanwhile, so one
+    // thread reads it for the whole CTA.
+    if (__syncthreads_or(threadIdx.x == 0 && ctrl->err != 0)) return;
     if (threadIdx.x < NBINS) {
         s_hist[threadIdx.x] = 0;
         s_max[threadIdx.x] = 0;

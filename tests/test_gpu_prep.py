@@ -111,3 +111,38 @@ def test_dense_list_from_both_ends(heavy):
     scale = oracle.backward(A.with_values(np.abs(A.values)), B.with_values(np.abs(B.values)), Ch, np.abs(d))
     for g, r, s in zip(got, want, scale):  # sums of at most 2000 terms: 2.2e-13 of their size
         assert np.all(np.abs(g.cpu().numpy() - r) <= 1e-12 * s)
+
+
+@pytest.mark.parametrize("what", ["row", "colptr", "a_rows_unchecked"])
+def test_malformed_operands_of_many_ctas(what):
+    """A fault that some CTAs report while others start (several waves of
+    them): every CTA takes the whole decision, and the next product is right."""
+    import torch
+    from paper_2303_02471_gb300 import ops
+    rng = np.random.default_rng(11)
+    n = 400003
+    A = _matrix(rng, 900, rng.integers(1, 5, 300), np.arange(0, 900, 3))
+    B = _matrix(rng, 300, np.where(np.arange(1000) % 50 == 0, 60, rng.integers(0, 4, 1000)))
+    # the 1000 columns over and over
+    reps = -(-n // 1000)
+    cp = (np.arange(reps)[:, None] * B.nnz + B.colptr[None, :-1]).ravel()
+    cp = np.append(cp, reps * B.nnz)
+    big = synth.CSC(300, reps * 1000, cp, np.tile(B.rowidx, reps), np.tile(B.values, reps))
+    dA, dB = upload(A), upload(big)
+    bad = ops.CscMatrix(dB.nrows, dB.ncols, dB.colptr.clone(), dB.rowidx.clone(), dB.values)
+    badA = ops.CscMatrix(dA.nrows, dA.ncols, dA.colptr, dA.rowidx.clone(), dA.values)
+    if what == "row":
+        bad.rowidx[3::50021] = 300
+    elif what == "colptr":
+        bad.colptr[1::10007] = -1
+    else:  # rows out of range without validation: found by the renumbering
+        badA.rowidx[::7] = 900
+    for _ in range(3):
+        with pytest.raises(RuntimeError, match="SPG_ERR_INVALID"):
+            if what.startswith("a_"):
+                ops.spgemm_symbolic(badA, dB, ops.Config(validate=False))
+            else:
+                ops.spgemm_symbolic(dA, bad)
+    C, plan = ops.spgemm(dA, upload(B))
+    plan.check()
+    assert_matches_oracle(C, A, B)
