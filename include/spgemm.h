@@ -313,7 +313,9 @@ spg_status spgemm_backward(spg_plan *plan, const spg_csc *A, const spg_csc *B,
  *   and returns the plan and the bytes of the slots; finish, once per plan and
  *   with the same A and B, writes C into `slots` (device, 256-byte aligned,
  *   kept by the caller while the plan is used), C_colptr and nnzC.  A plan
- *   whose finish failed serves only spg_plan_destroy.  Both synchronise.
+ *   that was not finished, or whose finish failed, serves spg_plan_destroy and
+ *   the queries of the preparation's counts; spgemm_numeric, spgemm_backward
+ *   and spgemm_single_pass_copy return SPG_ERR_INVALID.  Both synchronise.
  * spgemm_single_pass_copy: C's rows (device int32[nnzC]) and values (device,
  *   plan dtype) from the plan's slots, in order; asynchronous.  The values are
  *   those of the A and B given to spgemm_single_pass.

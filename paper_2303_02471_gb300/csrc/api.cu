@@ -139,6 +139,9 @@ struct spg_plan {
     Ctrl host{};
     BinOffsets off{};
     int64_t nnzC = 0;
+    // nnz(C) and the bins' statistics are there: the symbolic phase or the
+    // single pass has finished without an error
+    bool ready = false;
     Geo num_geo[NBINS];
     bool num_geo_ready = false;
     Geo bwd_geo[NBINS];
@@ -524,6 +527,7 @@ spg_status spgemm_symbolic(spg_handle *handle, const spg_csc *A, const spg_csc *
                                          P->L.scratch_ctas);
     }
     P->num_geo_ready = true;
+    P->ready = true;
     // the preparation, the scan with the control read, the bins
     P->sym_launches += std::max(1, scan_launches(P->nB)) + P->nonempty_bins();
     *nnzC = P->nnzC;
@@ -595,7 +599,7 @@ spg_status spgemm_numeric(spg_plan *P, const spg_csc *A, const spg_csc *B, const
                           int32_t *C_rowidx, void *C_values, spg_stream stream) {
     spg_status st = check_plan_operands(P, A, B);
     if (st != SPG_OK) return st;
-    if (!C_colptr || (P->nnzC > 0 && (!C_rowidx || !C_values))) return SPG_ERR_INVALID;
+    if (!P->ready || !C_colptr || (P->nnzC > 0 && (!C_rowidx || !C_values))) return SPG_ERR_INVALID;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     Ctrl *ctrl = P->ctrl();
     if (!P->reset_work(s)) return SPG_ERR_CUDA;
@@ -694,6 +698,7 @@ spg_status spgemm_single_pass_finish(spg_plan *P, const spg_csc *A, const spg_cs
     P->sym_launches += (P->nB > 0 ? 1 + scan_launches(P->nB) : 0) + P->nonempty_bins() +
                        std::max(1, scan_launches(P->nB));
     P->single = true;
+    P->ready = true;
     *nnzC = P->nnzC;
     return SPG_OK;
 }
@@ -734,7 +739,7 @@ spg_status spgemm_backward(spg_plan *P, const spg_csc *A, const spg_csc *B, cons
                            spg_stream stream) {
     spg_status st = check_plan_operands(P, A, B);
     if (st != SPG_OK) return st;
-    if (!C_colptr || (P->nnzC > 0 && (!C_rowidx || !dC_values))) return SPG_ERR_INVALID;
+    if (!P->ready || !C_colptr || (P->nnzC > 0 && (!C_rowidx || !dC_values))) return SPG_ERR_INVALID;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const size_t w = P->dtype == SPG_F64 ? 8 : 4;
     if (dA_values && P->nnzA > 0 && cudaMemsetAsync(dA_values, 0, (size_t)P->nnzA * w, s) != cudaSuccess)
