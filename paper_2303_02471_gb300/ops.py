@@ -381,7 +381,8 @@ def spgemm_single_pass(A: CscMatrix, B: CscMatrix, config: Optional[Config] = No
     the columns copied into C.  Returns (C, plan)."""
     config = config or Config()
     hd = lib_handle if lib_handle is not None else handle(A.device)
-    cA, cB = _csc(A), _csc(B, A.dtype)
+    # B's values are read here: they are described as what they are
+    cA, cB = _csc(A), _csc(B, A.dtype if B.values is None else None)
     colptr = torch.empty(B.ncols + 1, dtype=torch.int64, device=A.device)
     nnz = ctypes.c_int64()
     h = ctypes.c_void_p()
@@ -426,7 +427,7 @@ def spgemm_csr(A: CsrMatrix, B: CsrMatrix, config: Optional[Config] = None,
     config = config or Config()
     hd = lib_handle if lib_handle is not None else handle(A.device)
     cfg = config.native()
-    cA, cB = _csr(A), _csr(B, A.dtype)
+    cA, cB = _csr(A), _csr(B, A.dtype if B.values is None else None)
     nbytes = ctypes.c_size_t()
     N.check(N.lib().spgemm_csr_workspace_size(ctypes.byref(cA), ctypes.byref(cB), ctypes.byref(cfg),
                                               ctypes.byref(nbytes)), "spgemm_csr_workspace_size")

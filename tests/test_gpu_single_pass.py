@@ -72,3 +72,31 @@ def test_unfinished_plan_serves_no_product(handle):
     assert lib.spgemm_backward(h, ref, ref, _ptr(cp), _ptr(rows), _ptr(vals), _ptr(grad), None, s) == 0
     assert lib.spg_plan_check(h, s) == 0
     lib.spg_plan_destroy(h)
+
+
+@pytest.mark.parametrize("form", ["single_pass", "single_pass_workspace", "csr"])
+@pytest.mark.parametrize("a_is_double", [True, False])
+def test_operands_of_two_dtypes_are_refused(form, a_is_double):
+    """B's values are described by their own dtype, so that a B of the other
+    one is an error of the call instead of being read as A's."""
+    from paper_2303_02471_gb300 import ops
+    host = synth.rmat(8, seed=4, col_cap=60)
+    da, db = (np.float64, np.float32) if a_is_double else (np.float32, np.float64)
+    A, B = upload(host, da), upload(host, db)
+    if form == "csr":
+        A, B = (ops.CsrMatrix(M.ncols, M.nrows, M.colptr, M.rowidx, M.values) for M in (A, B))
+        call = ops.spgemm_csr
+    elif form == "single_pass":
+        call = ops.spgemm_single_pass
+    else:
+        import torch
+        need = ops.single_pass_workspace_size(A, B)
+
+        def call(a, b):
+            return ops.spgemm_single_pass(a, b, workspace=torch.empty(need, dtype=torch.uint8, device="cuda"))
+    with pytest.raises(RuntimeError, match="SPG_ERR_INVALID"):
+        call(A, B)
+    C, plan = call(A, A)
+    plan.check()
+    if form != "csr":
+        assert_matches_oracle(C, host, host)
