@@ -916,7 +916,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity, long l
 // writes map[r] (compact index or -1) and inv[compact] = r; k_row_remap
 // rewrites A's rows through map, reporting a row without a compact index
 // (kDetailRowMap).  mark: row_mark_bytes(m) zeroed bytes, 16-byte aligned;
-// counts: row_tile_count(m) ints.
+// counts: row_tile_count(m) ints (the tiles and their total).
 __global__ void k_check_rows(const int64_t *cp, const int32_t *row, int64_t nrows, int64_t ncols, int64_t nnz,
                              int validate, int64_t *mark, uint32_t *zlen, Ctrl *ctrl);
 size_t row_mark_bytes(int64_t m);

@@ -46,11 +46,14 @@ __global__ void __launch_bounds__(256) k_check_rows(const int64_t *__restrict__ 
 // (row_rule): map[r] = compact row or -1, inv[compact] = r.  ctrl->mrows =
 // their count.  A CTA takes a tile of kRowTile rows; the rows of the other
 // tiles are counted from the marks themselves up to kRowRecount tiles (which
-// saves a launch), else from the tiles' counts.  The marks are padded with
-// zeros to whole tiles.
+// saves a launch), up to kRowDirect tiles (8.4M rows) from the tiles' counts,
+// which every CTA then adds up (64 MB of L2 reads at the limit, growing with
+// the square of the tiles: 4.4 TB at 2^31 rows), else from their prefix
+// sums, a launch more.  The marks are padded with zeros to whole tiles.
 constexpr int kRowTile = 2048;
 constexpr int kRowThreads = 256;
 constexpr int kRowRecount = 8;
+constexpr int64_t kRowDirect = 4096;
 constexpr int kRowPer = kRowTile / kRowThreads;  // consecutive rows of a thread
 
 // The marks of thread threadIdx.x in tile `tile`, as bits.
@@ -75,8 +78,57 @@ __global__ void __launch_bounds__(kRowThreads) k_row_counts(const ulonglong2 *__
     if (threadIdx.x == 0) counts[blockIdx.x] = s_n;
 }
 
+// One CTA: the counts of `tiles` tiles into their exclusive prefix sums, the
+// total at counts[tiles] (at most the rows, so below 2^31).  kRowSumItems
+// consecutive counts a thread and step.
+constexpr int kRowSumThreads = 1024;
+constexpr int kRowSumItems = 8;
+
+__global__ void __launch_bounds__(kRowSumThreads) k_row_sums(int32_t *counts, int64_t tiles) {
+    __shared__ int s_warp[kRowSumThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int carry = 0;
+    for (int64_t base = 0; base < tiles; base += kRowSumThreads * kRowSumItems) {
+        const int64_t i0 = base + (int64_t)threadIdx.x * kRowSumItems;
+        int v[kRowSumItems];
+        int sum = 0;
+#pragma unroll
+        for (int u = 0; u < kRowSumItems; ++u) {
+            v[u] = i0 + u < tiles ? counts[i0 + u] : 0;
+            sum += v[u];
+        }
+        int incl = sum;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int o = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += o;
+        }
+        if (lane == 31) s_warp[warp] = incl;
+        __syncthreads();
+        int w = s_warp[lane];
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int o = __shfl_up_sync(0xffffffffu, w, d);
+            if (lane >= d) w += o;
+        }
+        const int total = __shfl_sync(0xffffffffu, w, 31);
+        const int before = __shfl_sync(0xffffffffu, w, warp > 0 ? warp - 1 : 0);
+        int run = carry + (warp > 0 ? before : 0) + incl - sum;
+#pragma unroll
+        for (int u = 0; u < kRowSumItems; ++u) {
+            if (i0 + u < tiles) counts[i0 + u] = run;
+            run += v[u];
+        }
+        carry += total;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) counts[tiles] = carry;
+}
+
+// counts: the tiles' counts, or (summed) their prefix sums and the total;
+// null: the tiles are counted here.
 __global__ void __launch_bounds__(kRowThreads) k_row_index(const ulonglong2 *__restrict__ marks, int64_t m,
-                                                          const int32_t *__restrict__ counts,
+                                                          const int32_t *__restrict__ counts, int summed,
                                                           int32_t *__restrict__ map, int32_t *__restrict__ inv,
                                                           Ctrl *ctrl) {
     __shared__ int s_warp[kRowThreads / 32];
@@ -86,7 +138,12 @@ __global__ void __launch_bounds__(kRowThreads) k_row_index(const ulonglong2 *__r
     __syncthreads();
     // rows with entries before the tile, and of all tiles
     int before = 0, all = 0;
-    if (counts) {
+    if (summed) {
+        if (threadIdx.x == 0) {
+            before = counts[blockIdx.x];
+            all = counts[gridDim.x];
+        }
+    } else if (counts) {
         for (int64_t i = threadIdx.x; i < gridDim.x; i += kRowThreads) {
             const int n = counts[i];
             all += n;
@@ -137,10 +194,12 @@ cudaError_t launch_row_index(const int64_t *mark, int64_t m, int32_t *counts, in
     const int64_t tiles = ceil_div(m, kRowTile);
     if (tiles <= 0) return cudaSuccess;
     const ulonglong2 *marks = reinterpret_cast<const ulonglong2 *>(mark);
-    const bool direct = tiles <= kRowRecount;
+    const bool direct = tiles <= kRowRecount, summed = tiles > kRowDirect;
     if (!direct) k_row_counts<<<(unsigned)tiles, kRowThreads, 0, s>>>(marks, counts);
-    k_row_index<<<(unsigned)tiles, kRowThreads, 0, s>>>(marks, m, direct ? nullptr : counts, map, inv, ctrl);
-    *launches += direct ? 1 : 2;
+    if (summed) k_row_sums<<<1, kRowSumThreads, 0, s>>>(counts, tiles);
+    k_row_index<<<(unsigned)tiles, kRowThreads, 0, s>>>(marks, m, direct ? nullptr : counts, summed ? 1 : 0, map, inv,
+                                                        ctrl);
+    *launches += direct ? 1 : summed ? 3 : 2;
     return cudaGetLastError();
 }
 

@@ -146,3 +146,25 @@ def test_malformed_operands_of_many_ctas(what):
     C, plan = ops.spgemm(dA, upload(B))
     plan.check()
     assert_matches_oracle(C, A, B)
+
+
+def test_rows_of_many_tiles():
+    """Row tiles at and past the number up to which every CTA adds up the
+    tiles' counts itself: the same rows, numbered with one launch more."""
+    from paper_2303_02471_gb300 import ops
+    rng = np.random.default_rng(3)
+    k, n = 3000, 200
+    za = rng.integers(1, 7, k)
+    launches = []
+    B = _matrix(rng, k, rng.integers(0, 40, n))
+    for tiles in (4096, 4097, 4096 + 8193):  # the last: more than one step of the prefix sums
+        m = tiles * 2048 - 5
+        cp = np.concatenate([[0], np.cumsum(za)]).astype(np.int64)
+        rows = np.concatenate([np.arange(z) * (m // z) + rng.integers(0, m // z, z) for z in za])
+        rows[0], rows[-1] = 0, m - 1  # the first and the last tile
+        A = synth.CSC(m, k, cp, rows.astype(np.int32), rng.standard_normal(rows.size))
+        C, plan = ops.spgemm(upload(A), upload(B))
+        plan.check()
+        assert_matches_oracle(C, A, B)
+        launches.append(plan.launch_count()["symbolic"])
+    assert launches[1] == launches[2] == launches[0] + 1
