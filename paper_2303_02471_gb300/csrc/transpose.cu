@@ -134,6 +134,11 @@ __global__ void __launch_bounds__(256) k_tr_sort_warp(const int64_t *__restrict_
 // A CTA looks through blockDim columns at a time, one per thread, dealt over
 // the CTAs by index so that neighbouring long columns go to different CTAs;
 // where there are none (the common case) one round of loads is all it does.
+// Its grid (sort_cta_grid): a CTA per 64 columns, which keeps that round
+// short, or a CTA per column that can be long (at most nnz / 257 are) where
+// that is more, up to four CTAs per SM, whose share of the long columns is
+// even enough (64 rows of 10000 entries: 0.74 ms, one of them alone 0.53,
+// all 64 in one CTA 29.8).
 __global__ void __launch_bounds__(512) k_tr_sort_cta(const int64_t *__restrict__ Tcp, int64_t ncolsT, int32_t *Trow,
                                                     int64_t *Tperm, int32_t *gkey, int64_t *gval) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -188,6 +193,11 @@ __global__ void __launch_bounds__(512) k_tr_sort_cta(const int64_t *__restrict__
         }
         __syncthreads();
     }
+}
+
+int sort_cta_grid(int64_t m, int64_t nnz, int sms) {
+    const int64_t longest = std::min<int64_t>(m, nnz / 257);
+    return (int)std::max<int64_t>(1, std::min<int64_t>(std::max<int64_t>(ceil_div(m, 64), longest), 4 * (int64_t)sms));
 }
 
 // T's values through the permutation, for the entries T actually holds.
@@ -276,7 +286,11 @@ spg_status spg_csc_transpose(const spg_csc *M, int64_t *T_colptr, int32_t *T_row
         k_tr_sort_warp<<<(unsigned)ceil_div(m, 256), 256, 0, s>>>(T_colptr, m, T_rowidx, pm);
         const size_t smem = (size_t)kTrSmemSort * 12;
         cudaFuncSetAttribute(k_tr_sort_cta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_tr_sort_cta<<<(unsigned)std::min<int64_t>(ceil_div(m, 64), 608), 512, smem, s>>>(
+        int dev = 0, sms = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            return SPG_ERR_CUDA;
+        k_tr_sort_cta<<<(unsigned)sort_cta_grid(m, nnz, sms), 512, smem, s>>>(
             T_colptr, m, T_rowidx, pm, reinterpret_cast<int32_t *>(ws + L.key),
             reinterpret_cast<int64_t *>(ws + L.val));
         if (T_values) {

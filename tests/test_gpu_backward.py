@@ -336,3 +336,38 @@ def test_transpose_row_lengths(lengths):
     assert np.array_equal(Th.rowidx, R.rowidx)
     assert np.array_equal(Th.values, R.values)
     assert np.array_equal(perm.cpu().numpy(), q)
+
+
+def _time_ms(call, reps=7):
+    import torch
+    call()
+    times = []
+    for _ in range(reps):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        call()
+        b.record()
+        b.synchronize()
+        times.append(a.elapsed_time(b))
+    return sorted(times)[reps // 2]
+
+
+def _long_rows(m, n, length):
+    """m rows of `length` entries, in columns dealt from a shifted stride."""
+    k = np.arange(length)
+    cols = np.concatenate([(k * (n // length) + 7 * i) % n for i in range(m)])
+    rows = np.repeat(np.arange(m), length)
+    return synth.from_coo(m, n, rows, cols, np.random.default_rng(m).standard_normal(rows.size))
+
+
+def test_transpose_spreads_few_long_rows():
+    """64 rows of 10000 entries are sorted beside one another: a single one
+    takes a CTA the same time (the bound allows four times that, and one CTA
+    for all 64 would take 50 times)."""
+    from paper_2303_02471_gb300 import ops
+    one, many = (upload(_long_rows(m, 20000, 10000)) for m in (1, 64))
+    T, perm = ops.csc_transpose(many)
+    R, q = oracle.transpose(_long_rows(64, 20000, 10000))
+    assert np.array_equal(T.rowidx.cpu().numpy(), R.rowidx)
+    assert np.array_equal(perm.cpu().numpy(), q)
+    assert _time_ms(lambda: ops.csc_transpose(many)) < 4 * _time_ms(lambda: ops.csc_transpose(one))
