@@ -45,12 +45,12 @@ __global__ void k_tr_scatter(const int64_t *__restrict__ cp, const int32_t *__re
     }
 }
 
-// Output columns of at most 256 entries, 32 per warp.  A lane sorts its own
-// column of up to kLaneSort entries with a sorting network in registers (of
-// the smallest size that fits the warp's columns); the whole warp then sorts
-// the longer ones one after another.  Grid columns and stencils have only
-// columns of a few entries, and a warp per column spent a 256-entry network
-// on each: 226 us for the 64000 rows of a 40^3 prolongation.
+// Output columns of at most 256 entries, `per` of them per warp.  A lane sorts
+// its own column of up to kLaneSort entries with a sorting network in registers
+// (of the smallest size that fits the warp's columns); the whole warp then
+// sorts the longer ones one after another.  Grid columns and stencils have
+// only columns of a few entries, and a warp per column spent a 256-entry
+// network on each: 226 us for the 64000 rows of a 40^3 prolongation.
 constexpr int kLaneSort = 8;
 
 template <int N>
@@ -103,11 +103,12 @@ __device__ __forceinline__ void warp_sort(int64_t b, int L, int32_t *Trow, int64
     }
 }
 
-__global__ void __launch_bounds__(256) k_tr_sort_warp(const int64_t *__restrict__ Tcp, int64_t ncolsT, int32_t *Trow,
-                                                     int64_t *Tperm) {
-    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(256) k_tr_sort_warp(const int64_t *__restrict__ Tcp, int64_t ncolsT, int per,
+                                                     int32_t *Trow, int64_t *Tperm) {
+    const int lane = threadIdx.x & 31;
+    const int64_t c = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per + lane;
     int64_t b = 0, len = 0;
-    if (c < ncolsT) {
+    if (lane < per && c < ncolsT) {
         b = Tcp[c];
         len = Tcp[c + 1] - b;
     }
@@ -193,6 +194,21 @@ __global__ void __launch_bounds__(512) k_tr_sort_cta(const int64_t *__restrict__
         }
         __syncthreads();
     }
+}
+
+// Columns per warp of k_tr_sort_warp: 32 where that gives every warp slot of
+// the chip a warp (kSortWarps per SM), else fewer, so that longer columns are
+// not left to the few warps of a matrix with few columns.  Whole transposes:
+// 64 rows of 200 entries 1018 us with 32 columns per warp, 92 so; 100000 rows
+// of 100 1405 and 1184, R-MAT 2^16 773 and 384; the 40^3 prolongation 77 and
+// 80, 200000 rows of 3 entries with one of 200 in 64 191 and 219 (a warp per
+// column: 1467).
+constexpr int kSortWarps = 64;
+
+int sort_warp_columns(int64_t m, int sms) {
+    int per = 32;
+    while (per > 1 && ceil_div(m, per) < kSortWarps * (int64_t)sms) per >>= 1;
+    return per;
 }
 
 int sort_cta_grid(int64_t m, int64_t nnz, int sms) {
@@ -283,13 +299,14 @@ spg_status spg_csc_transpose(const spg_csc *M, int64_t *T_colptr, int32_t *T_row
     if (nnz > 0) {
         const int gc = (int)std::min<int64_t>(ceil_div(M->ncols * kScatterLanes, 256), 4096);
         k_tr_scatter<<<gc, 256, 0, s>>>(M->colptr, M->rowidx, M->ncols, m, cnt, T_rowidx, pm);
-        k_tr_sort_warp<<<(unsigned)ceil_div(m, 256), 256, 0, s>>>(T_colptr, m, T_rowidx, pm);
-        const size_t smem = (size_t)kTrSmemSort * 12;
-        cudaFuncSetAttribute(k_tr_sort_cta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         int dev = 0, sms = 0;
         if (cudaGetDevice(&dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
             return SPG_ERR_CUDA;
+        const int per = sort_warp_columns(m, sms);
+        k_tr_sort_warp<<<(unsigned)ceil_div(m, 8 * per), 256, 0, s>>>(T_colptr, m, per, T_rowidx, pm);
+        const size_t smem = (size_t)kTrSmemSort * 12;
+        cudaFuncSetAttribute(k_tr_sort_cta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         k_tr_sort_cta<<<(unsigned)sort_cta_grid(m, nnz, sms), 512, smem, s>>>(
             T_colptr, m, T_rowidx, pm, reinterpret_cast<int32_t *>(ws + L.key),
             reinterpret_cast<int64_t *>(ws + L.val));

@@ -371,3 +371,20 @@ def test_transpose_spreads_few_long_rows():
     assert np.array_equal(T.rowidx.cpu().numpy(), R.rowidx)
     assert np.array_equal(perm.cpu().numpy(), q)
     assert _time_ms(lambda: ops.csc_transpose(many)) < 4 * _time_ms(lambda: ops.csc_transpose(one))
+
+
+@pytest.mark.parametrize("m", [1, 31, 64, 1000])
+def test_transpose_spreads_few_rows_of_a_warp_sort(m):
+    """Few rows of 200 entries, each sorted by a warp, go to many warps: a
+    thousand take less than four times as long as one (a warp for 32 of them
+    took eight times)."""
+    from paper_2303_02471_gb300 import ops
+    M = _long_rows(m, 4000, 200)
+    d = upload(M)
+    T, perm = ops.csc_transpose(d)
+    R, q = oracle.transpose(M)
+    assert np.array_equal(T.colptr.cpu().numpy(), R.colptr)
+    assert np.array_equal(T.rowidx.cpu().numpy(), R.rowidx)
+    assert np.array_equal(perm.cpu().numpy(), q)
+    one = upload(_long_rows(1, 4000, 200))
+    assert _time_ms(lambda: ops.csc_transpose(d)) < 4 * _time_ms(lambda: ops.csc_transpose(one))
