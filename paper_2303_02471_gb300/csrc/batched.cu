@@ -7,7 +7,7 @@
 //   * a group item is blockDim / G columns of a warp-group bin;
 //   * when no product has more than 32 * kWarpDenseWords rows, a dense item
 //     is blockDim / 32 columns of the dense bin, one per warp (in the
-//     backward, CTA-level columns of up to kWarpBackwardOps products).
+//     backward, all CTA-level columns, where none holds the launch up).
 // Items are ordered heaviest first (dense, then CTA bins from the largest,
 // then the group bins), the GPU form of processing columns by decreasing
 // Op_j (Section 3.1).  Per-column work is the same device code as the
@@ -283,8 +283,12 @@ __device__ __forceinline__ ItemRef item_ref(const BItems &it, int64_t item) {
 // and warp-level synchronisation only: the column's fixed cost (clearing,
 // prefix, extraction) is small and no CTA barrier is paid per column.
 constexpr int64_t kWarpDenseWords = 1024;
-// Largest Op_j of a column that one warp takes in the backward.
-constexpr int64_t kWarpBackwardOps = 8192;
+// The backward works columns in warps where the longest has at most one in
+// kWarpBackwardShare * SMs of the products of all.
+constexpr int kWarpBackwardShare = 10;
+// Threads of a CTA that works one column of the backward at a time, where
+// there are many.
+constexpr int kBackwardThreads = 256;
 
 // Position of row among the flagged rows of its column: the word's prefix
 // count plus the flags below it in the word.
@@ -389,11 +393,24 @@ __device__ __forceinline__ bool warp_dense_numeric(const TOps<VT> &o, int32_t j,
 }
 
 // Backward of column j in one warp: C's rows set the flags, whose prefix
-// counts give the position of dC_ij; then S lanes walk each B entry's A column
-// (S the largest power of two with S times the column's entries at most 32),
-// so a * dC_ij is summed in a register and log2(S) shuffles end an entry, and
-// no search for a product's owner is needed.  Each entry of dB belongs to one
-// column: it is stored.
+// counts give the position of dC_ij.  The column's B entries are taken 32 at a
+// time, one per lane, and their A columns walked
+//   * of more than kWarpEntry products: by the whole warp, one after another;
+//   * the others: by S lanes each, S the smallest power of two with which an
+//     entry of the average length takes at most kWarpRounds rounds, and no lane
+//     is idle for want of entries.
+// So a * dC_ij is summed in a register and log2(S) shuffles end an entry, no
+// search for a product's owner is needed, an entry's lanes take neighbouring
+// products (the adds to dA of one sector travel together), and a long entry
+// among short ones holds no lane up.  Lanes dealt by the number of entries
+// alone (one lane each from 17 on) took 1276 us for four products of 600
+// columns with one entry of 4000 products and 19 of 4 (188 so; 309 with a
+// 512-thread CTA per column), 255 with 20 entries of 204 (173), and 2160 for 48
+// products of matrices of equal columns (1489).  Each entry of dB belongs to
+// one column: it is stored.
+constexpr int kWarpEntry = 64;
+constexpr int kWarpRounds = 2;
+
 template <typename VT>
 __device__ __forceinline__ void warp_dense_backward(const TOps<VT> &o, int32_t j, int64_t c0, int64_t nn,
                                                     const int32_t *Crow, const VT *dC, uint2 *bm, int W, VT *dA,
@@ -409,27 +426,16 @@ __device__ __forceinline__ void warp_dense_backward(const TOps<VT> &o, int32_t j
     warp_dense_prefix(bm, W);
     const VT *gdc = dC + c0;
     const int64_t p0 = o.Bcp[j], p1 = o.Bcp[j + 1];
-    int S = 32;
-    while (S > 1 && (p1 - p0) * S > 32) S >>= 1;
-    const int sub = lane / S, sl = lane & (S - 1), per = 32 / S;
     constexpr int U = 4;  // products a lane gathers at once
-    for (int64_t pb = p0; pb < p1; pb += per) {
-        const int64_t p = pb + sub;
-        int z = 0;
-        int64_t a0 = 0;
-        VT b = VT(0), acc = VT(0);
-        if (p < p1) {
-            const int32_t k = o.Brow[p];
-            a0 = o.Acp[k];
-            z = (int)(o.Acp[k + 1] - a0);
-            b = o.Bval[p];
-        }
-        for (int q0 = sl; q0 < z; q0 += U * S) {
+    // a lane's part of an entry: products first, first + step, ...
+    auto walk = [&](int64_t a0, int z, VT b, int first, int step) -> VT {
+        VT acc = VT(0);
+        for (int q0 = first; q0 < z; q0 += U * step) {
             int32_t row[U];
             VT av[U], g[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                const int q = q0 + u * S;
+                const int q = q0 + u * step;
                 row[u] = q < z ? o.Arow[a0 + q] : -1;
                 av[u] = q < z ? o.Aval[a0 + q] : VT(0);
             }
@@ -437,13 +443,45 @@ __device__ __forceinline__ void warp_dense_backward(const TOps<VT> &o, int32_t j
             for (int u = 0; u < U; ++u) g[u] = row[u] >= 0 ? gdc[warp_dense_rank(bm, row[u])] : VT(0);
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                if (row[u] >= 0 && dA) atomicAdd(&dA[a0 + q0 + u * S], b * g[u]);
+                if (row[u] >= 0 && dA) atomicAdd(&dA[a0 + q0 + u * step], b * g[u]);
                 acc += av[u] * g[u];
             }
         }
         __syncwarp();
-        for (int d = S >> 1; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
-        if (dB && sl == 0 && p < p1) dB[p] = acc;
+        return acc;
+    };
+    for (int64_t pb = p0; pb < p1; pb += 32) {
+        const int ne = (int)(p1 - pb < 32 ? p1 - pb : 32);
+        int z = 0;
+        int64_t a0 = 0;
+        VT b = VT(0);
+        if (lane < ne) {
+            const int32_t k = o.Brow[pb + lane];
+            a0 = o.Acp[k];
+            z = (int)(o.Acp[k + 1] - a0);
+            b = o.Bval[pb + lane];
+        }
+        const unsigned lng = __ballot_sync(0xffffffffu, z > kWarpEntry);
+        for (unsigned todo = lng; todo; todo &= todo - 1u) {
+            const int s = __ffs(todo) - 1;
+            VT acc = walk(__shfl_sync(0xffffffffu, a0, s), __shfl_sync(0xffffffffu, z, s),
+                          __shfl_sync(0xffffffffu, b, s), lane, 32);
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
+            if (dB && lane == 0) dB[pb + s] = acc;
+        }
+        const int zs = z > kWarpEntry ? 0 : z;
+        const int total = (int)__reduce_add_sync(0xffffffffu, (unsigned)zs);
+        int S = 1;
+        while (S < 32 && (kWarpRounds * U * S * ne < total || 2 * S * ne <= 32)) S <<= 1;
+        const int sl = lane & (S - 1);
+        for (int i = 0; i < ne; i += 32 / S) {
+            const int e = i + lane / S;
+            VT acc = walk(__shfl_sync(0xffffffffu, a0, e), __shfl_sync(0xffffffffu, zs, e),
+                          __shfl_sync(0xffffffffu, b, e), sl, S);
+            for (int d = S >> 1; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
+            if (dB && sl == 0 && e < ne && !(lng >> e & 1u)) dB[pb + e] = acc;
+        }
     }
 }
 
@@ -818,20 +856,43 @@ namespace {
 
 // Dense columns of the forward phases are worked one per warp when every
 // product's flags fit kWarpDenseWords words.  So are the CTA-level columns of
-// the backward where in addition no column is long enough to hold the launch
-// up on one warp and the warps' flags leave room for two CTAs per SM (a
-// batch step of 12 products of 300 to 4000 rows, forward and backward: 716 us
-// with one 512-thread CTA per column in the backward, 784 us with its walk
-// split into long and short entries, 686 us with one warp per column).
+// the backward where in addition no column holds the launch up on one warp and
+// the warps' flags leave room for two CTAs per SM.  All products' sum over the
+// longest column's, and the backward's time with one column per warp and per
+// CTA (double, us): 20 columns of 8000 alone 20, 227 and 64; R-MAT 2^10 to 2^13,
+// 8 of each, 487, 218 and 182; 821, 313 and 282; 1248, 520 and 488; 1302, 1343
+// and 1060; R-MAT 2^12 of fewer products 1756, 245 and 313; 12000 columns of
+// 600 12000, 161 and 361.
 bool warp_dense(const spg_bplan &P, int phase) {
     if (P.Wmax > kWarpDenseWords) return false;
     if (phase < 2) return P.host.hist[BIN_DENSE] != 0;
-    bool any = false;
+    unsigned long long most = 0, all = 0;
     for (int b = BIN_CTA0; b < NBINS; ++b) {
-        any |= P.host.hist[b] != 0;
-        if (P.host.maxop[b] > (unsigned long long)kWarpBackwardOps) return false;
+        most = std::max(most, P.host.maxop[b]);
+        all += P.host.binprod[b];
     }
-    return any && (size_t)(P.threads / 32) * al16((size_t)P.Wmax * 8) <= P.smem_optin / 2;
+    if (most * (unsigned long long)(kWarpBackwardShare * P.sms) > all) return false;
+    return most > 0 && (size_t)(P.threads / 32) * al16((size_t)P.Wmax * 8) <= P.smem_optin / 2;
+}
+
+// Shared memory that a CTA of the backward's one-column form cannot do without:
+// the walk's scratch and the flags.
+size_t backward_fixed(const spg_bplan &P, int threads) {
+    const size_t walk = P.any_f64 ? walk_smem_bytes<double>(threads) : walk_smem_bytes<float>(threads);
+    return walk + al16((size_t)threads * 4) + al16((size_t)P.Wmax * 8);
+}
+
+// Threads per CTA of a phase.  The backward with a column per CTA: 256, as in
+// the single product's (more CTAs overlap one another's per-column barriers),
+// where four such CTAs fit an SM and the columns outnumber the CTAs of the
+// configured size (four products of 3000 columns of 600 products in 40000
+// rows: 531 us with 512 threads, 355 with 256; 20 columns of 8000: 82 and 107).
+int phase_threads(const spg_bplan &P, int phase) {
+    if (phase < 2 || P.threads <= kBackwardThreads || warp_dense(P, phase)) return P.threads;
+    int64_t columns = 0;
+    for (int b = BIN_CTA0; b < NBINS; ++b) columns += (int64_t)P.host.hist[b];
+    return columns > 2 * (int64_t)P.sms && 4 * backward_fixed(P, kBackwardThreads) <= P.smem_optin ? kBackwardThreads
+                                                                                                   : P.threads;
 }
 
 // Items of a phase, heaviest first.
@@ -890,17 +951,22 @@ size_t phase_smem(const spg_bplan &P, int phase, int threads, int64_t &cap_cta, 
         cap_dense = 0;
         return need;
     }
-    const size_t fixed = walk + (phase == 2 ? al16((size_t)threads * 4) : 0) + al16((size_t)P.Wmax * 8);
-    const size_t room = P.smem_optin > fixed ? P.smem_optin - fixed : 0;
     cap_dense = 0;
     if (phase == 2) {
-        // CTA-level columns of the backward all use the dense lookup
+        // CTA-level columns of the backward all use the dense lookup; dC of a
+        // column in what a CTA's share of the SM leaves (kSmemReserve: what
+        // the runtime and the kernel's static arrays take)
+        constexpr size_t kSmemReserve = 2048;
+        const size_t fixed = backward_fixed(P, threads);
+        const size_t ctas = std::max<size_t>(1, std::min<size_t>(1024 / threads, P.smem_optin / (fixed + kSmemReserve)));
+        const size_t share = P.smem_optin / ctas;
         int64_t mx = (int64_t)P.host.maxnnz[BIN_DENSE];
         for (int c = 0; c < kNumCtaBins; ++c) mx = std::max<int64_t>(mx, (int64_t)P.host.maxnnz[BIN_CTA0 + c]);
-        cap_dense = std::min<int64_t>((int64_t)(room / w), mx);
+        if (share > fixed + kSmemReserve) cap_dense = std::min<int64_t>((int64_t)((share - fixed - kSmemReserve) / w), mx);
         if ((cta || dense) && !wd) need = std::max(need, fixed + (size_t)cap_dense * w);
         return need;
     }
+    const size_t fixed = walk + al16((size_t)P.Wmax * 8);
     if (dense) need = std::max(need, fixed);
     if (cta)
         need = std::max(need, walk + (P.any_f64 ? cta_table_bytes<double>(cap_cta) : cta_table_bytes<float>(cap_cta)) +
@@ -920,12 +986,13 @@ struct PhaseLaunch {
     BTask b;
     BItems it;
     size_t smem = 0;
-    int grid = 0;
+    int grid = 0, threads = 0;
 };
 
 spg_status prepare_phase(spg_bplan &P, int phase, PhaseLaunch &L) {
     int64_t cap_cta = 0, cap_dense = 0, cap_sym = 0;
-    const int threads = P.threads;
+    const int threads = phase_threads(P, phase);
+    L.threads = threads;
     L.smem = phase_smem(P, phase, threads, cap_cta, cap_dense, cap_sym);
     if (L.smem > P.smem_optin) return SPG_ERR_UNSUPPORTED;
     L.b = P.task();
@@ -948,9 +1015,9 @@ spg_status prepare_phase(spg_bplan &P, int phase, PhaseLaunch &L) {
 spg_status enqueue_phase(const spg_bplan &P, int phase, const PhaseLaunch &L, cudaStream_t s) {
     if (cudaMemsetAsync(L.b.counter, 0, sizeof(unsigned long long), s) != cudaSuccess) return SPG_ERR_CUDA;
     if (L.it.nitems == 0) return SPG_OK;
-    if (phase == 0) k_batched<0><<<L.grid, P.threads, L.smem, s>>>(L.b, L.it);
-    else if (phase == 1) k_batched<1><<<L.grid, P.threads, L.smem, s>>>(L.b, L.it);
-    else k_batched<2><<<L.grid, P.threads, L.smem, s>>>(L.b, L.it);
+    if (phase == 0) k_batched<0><<<L.grid, L.threads, L.smem, s>>>(L.b, L.it);
+    else if (phase == 1) k_batched<1><<<L.grid, L.threads, L.smem, s>>>(L.b, L.it);
+    else k_batched<2><<<L.grid, L.threads, L.smem, s>>>(L.b, L.it);
     return cudaGetLastError() == cudaSuccess ? SPG_OK : SPG_ERR_CUDA;
 }
 

@@ -269,3 +269,70 @@ def test_product_autotune_chooses_and_caches(tmp_path):
     C, plan = ops.spgemm_single_pass(dA, dA, cfg3)
     plan.check()
     assert_matches_oracle(C, A, A)
+
+
+def _matrix(rng, nrows, lengths, dtype=np.float64):
+    cp = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int64)
+    rows = np.concatenate([rng.permutation(nrows)[:n] for n in lengths]).astype(np.int32)
+    return synth.CSC(nrows, len(lengths), cp, rows, rng.standard_normal(rows.size).astype(dtype))
+
+
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+def test_batched_backward_entry_lengths_per_warp(dtype):
+    """Entries at the edges of the warp's split (by the whole warp above 64
+    products, by 1 to 32 lanes below) in columns of 1 to 70 entries, enough of
+    them that the batch's backward works a column per warp.  The longest sum
+    (dA) has 6000 terms: 6000 u = 3.6e-4 in float, 6.7e-13 in double."""
+    import torch
+    from paper_2303_02471_gb300 import ops
+    rng = np.random.default_rng(23)
+    n, m, k = 6000, 1037, 70
+    za = np.array([[0, 1, 2, 7, 8, 9, 31, 32, 33, 63, 64, 65, 127, 128, 129, 300][i % 16] for i in range(k)])
+    A = _matrix(rng, m, za, dtype)
+    B = _matrix(rng, k, np.arange(n) % 70 + 1, dtype)
+    op = np.add.reduceat(za[B.rowidx], B.colptr[:-1])
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert op.max() * 10 * sms <= op.sum()
+    dA, dB = upload(A, dtype), upload(B, dtype)
+    Cs, plan = ops.spgemm_batched([dA], [dB], ops.Config(t=1))
+    dc = torch.as_tensor(rng.standard_normal(Cs[0].nnz).astype(dtype), device="cuda")
+    full = ops.spgemm_batched_backward(plan, [dA], [dB], Cs, [dc])
+    only_b = ops.spgemm_batched_backward(plan, [dA], [dB], Cs, [dc], need_dA=False)
+    only_a = ops.spgemm_batched_backward(plan, [dA], [dB], Cs, [dc], need_dB=False)
+    plan.check()
+    assert only_b[0] is None and only_a[1] is None
+    Ch, d = Cs[0].to_host(), dc.cpu().numpy()
+    want = oracle.backward(A, B, Ch, d)
+    scale = oracle.backward(A.with_values(np.abs(A.values)), B.with_values(np.abs(B.values)), Ch, np.abs(d))
+    tau = 1e-12 if dtype == np.float64 else 6000 * 2.0 ** -24
+    for got, r, s in ((full[0][0], want[0], scale[0]), (full[1][0], want[1], scale[1]),
+                      (only_a[0][0], want[0], scale[0]), (only_b[1][0], want[1], scale[1])):
+        assert np.all(np.abs(got.cpu().numpy().astype(np.float64) - r) <= tau * s)
+
+
+def test_batched_backward_of_skewed_columns_keeps_pace():
+    """Columns of one entry of 4000 products and 19 of 4 against columns of 20
+    entries of 204: as many products, and as many adds to each place of dA
+    (measured equal within a tenth; one lane walking the long entry took 4.6
+    times as long)."""
+    import torch
+    from paper_2303_02471_gb300 import ops
+    rng = np.random.default_rng(1)
+
+    def backward_ms(za):
+        A, B = upload(_matrix(rng, 5000, za)), upload(_matrix(rng, 20, np.full(600, 20)))
+        As, Bs = [A] * 4, [B] * 4
+        Cs, plan = ops.spgemm_batched(As, Bs)
+        dCs = [torch.randn(C.nnz, dtype=torch.float64, device="cuda") for C in Cs]
+        times = []
+        for _ in range(9):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            ops.spgemm_batched_backward(plan, As, Bs, Cs, dCs)
+            b.record()
+            b.synchronize()
+            times.append(a.elapsed_time(b))
+        plan.check()
+        return sorted(times)[4]
+
+    assert backward_ms(np.array([4000] + [4] * 19)) < 2.5 * backward_ms(np.full(20, 204))
