@@ -1276,6 +1276,7 @@ spg_status spgemm_batched_backward(spg_bplan *P, const spg_csc *A, const spg_csc
         BProb &q = P->prob[i];
         if (P->nnz[i] > 0 && (!C_rowidx[i] || !dC_values[i])) return SPG_ERR_INVALID;
         q.Aval = A[i].values; q.Bval = B[i].values;
+        q.Acp = A[i].colptr; q.Arow = A[i].rowidx; q.Bcp = B[i].colptr; q.Brow = B[i].rowidx;
         q.Crow = const_cast<int32_t *>(C_rowidx[i]);
         q.dC = dC_values[i];
         q.dA = dA_values ? dA_values[i] : nullptr;

@@ -336,3 +336,27 @@ def test_batched_backward_of_skewed_columns_keeps_pace():
         return sorted(times)[4]
 
     assert backward_ms(np.array([4000] + [4] * 19)) < 2.5 * backward_ms(np.full(20, 204))
+
+
+def test_batched_backward_reads_the_operands_it_is_given():
+    """The same patterns in other buffers than the forward's, whose rows are
+    overwritten meanwhile: nothing of the forward's operands is read."""
+    import torch
+    from paper_2303_02471_gb300 import ops
+    pairs = synth.batch_pairs(6, seed=9, n_scale=0.05)
+    As, Bs = _upload_pairs(pairs)
+    Cs, plan = ops.spgemm_batched(As, Bs)
+    dCs = [torch.randn(C.nnz, dtype=C.values.dtype, device="cuda") for C in Cs]
+    want = ops.spgemm_batched_backward(plan, As, Bs, Cs, dCs)
+
+    def copy(M):
+        return ops.CscMatrix(M.nrows, M.ncols, M.colptr.clone(), M.rowidx.clone(), M.values.clone())
+    As2, Bs2 = [copy(M) for M in As], [copy(M) for M in Bs]
+    for M in As + Bs:
+        M.rowidx.zero_()
+    got = ops.spgemm_batched_backward(plan, As2, Bs2, Cs, dCs)
+    plan.check()
+    for g, w in zip(got[0] + got[1], want[0] + want[1]):
+        # sums of at most 1600 terms in another order, in scale with the largest
+        tau = 1600 * torch.finfo(w.dtype).eps
+        assert (g - w).abs().max() <= tau * 40 * w.abs().max()
