@@ -811,6 +811,7 @@ struct spg_bplan {
     int64_t ntot = 0, ncp = 0, na = 0, nbe = 0;
     std::vector<BProb> prob;  // host copy of the problem table
     std::vector<int64_t> nnz;
+    std::vector<int64_t> nnzA, nnzB;  // entries of the operands the batch was planned for
     Ctrl host{};
     BinOffsets off{};
     int64_t Wmax = 0, mmax = 0;
@@ -1100,6 +1101,8 @@ spg_status spgemm_batched_symbolic(spg_handle *handle, int32_t nb, const spg_csc
     std::vector<int64_t> col0s(nb + 1), segs(nb + 1), aoff(nb + 1), boffe(nb + 1), acol0(nb + 1);
     std::vector<VMat> vA(nb), vB(nb);
     P->prob.resize(nb);
+    P->nnzA.resize(nb);
+    P->nnzB.resize(nb);
     int64_t ntot = 0, ncp = 0, na = 0, nbe = 0, ntotA = 0;
     for (int i = 0; i < nb; ++i) {
         col0s[i] = ntot;
@@ -1117,6 +1120,8 @@ spg_status spgemm_batched_symbolic(spg_handle *handle, int32_t nb, const spg_csc
         q.dtype = A[i].dtype;
         vA[i] = VMat{A[i].colptr, A[i].rowidx, A[i].nrows, A[i].ncols, A[i].nnz, ntotA};
         vB[i] = VMat{B[i].colptr, B[i].rowidx, B[i].nrows, B[i].ncols, B[i].nnz, ntot};
+        P->nnzA[i] = A[i].nnz;
+        P->nnzB[i] = B[i].nnz;
         if (A[i].dtype == SPG_F64) P->any_f64 = true;
         P->mmax = std::max<int64_t>(P->mmax, A[i].nrows);
         ntot += B[i].ncols;
@@ -1205,10 +1210,12 @@ spg_status spgemm_batched_symbolic(spg_handle *handle, int32_t nb, const spg_csc
 
 static spg_status batch_matches(const spg_bplan *P, const spg_csc *A, const spg_csc *B) {
     if (!P) return SPG_ERR_INVALID;
-    if (P->nb > 0 && (!A || !B)) return SPG_ERR_INVALID;
+    const spg_status st = check_batch(P->nb, A, B);
+    if (st != SPG_OK) return st;
     for (int i = 0; i < P->nb; ++i) {
         const BProb &q = P->prob[i];
         if (A[i].nrows != q.m || B[i].ncols != q.n || A[i].dtype != q.dtype || B[i].dtype != q.dtype) return SPG_ERR_INVALID;
+        if (A[i].nnz != P->nnzA[i] || B[i].nnz != P->nnzB[i]) return SPG_ERR_INVALID;
         if ((A[i].nnz > 0 && !A[i].values) || (B[i].nnz > 0 && !B[i].values)) return SPG_ERR_INVALID;
     }
     return SPG_OK;

@@ -360,3 +360,27 @@ def test_batched_backward_reads_the_operands_it_is_given():
         # sums of at most 1600 terms in another order, in scale with the largest
         tau = 1600 * torch.finfo(w.dtype).eps
         assert (g - w).abs().max() <= tau * 40 * w.abs().max()
+
+
+def test_batched_plan_refuses_operands_of_other_sizes():
+    """Numeric and backward compare the operands' entries with the plan's, as
+    the single product does: the gradients are zeroed by the plan's counts."""
+    import torch
+    from paper_2303_02471_gb300 import ops
+    pairs = synth.batch_pairs(4, seed=2, n_scale=0.05)
+    As, Bs = _upload_pairs(pairs)
+    Cs, plan = ops.spgemm_batched(As, Bs)
+    dCs = [torch.ones_like(C.values) for C in Cs]
+
+    def shorter(M):  # one entry less in the last column
+        cp = M.colptr.clone()
+        cp[-1] -= 1
+        return ops.CscMatrix(M.nrows, M.ncols, cp, M.rowidx[:-1].clone(), M.values[:-1].clone())
+    for a, b in (([shorter(As[0])] + As[1:], Bs), (As, Bs[:-1] + [shorter(Bs[-1])])):
+        with pytest.raises(RuntimeError, match="SPG_ERR_INVALID"):
+            ops.spgemm_batched_numeric(plan, a, b)
+        with pytest.raises(RuntimeError, match="SPG_ERR_INVALID"):
+            ops.spgemm_batched_backward(plan, a, b, Cs, dCs)
+    for (A, B), C in zip(pairs, ops.spgemm_batched_numeric(plan, As, Bs)):
+        assert_matches_oracle(C, A, B)
+    plan.check()
