@@ -388,3 +388,38 @@ def test_transpose_spreads_few_rows_of_a_warp_sort(m):
     assert np.array_equal(perm.cpu().numpy(), q)
     one = upload(_long_rows(1, 4000, 200))
     assert _time_ms(lambda: ops.csc_transpose(d)) < 4 * _time_ms(lambda: ops.csc_transpose(one))
+
+
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+@pytest.mark.parametrize("tall", [False, True])
+def test_backward_entry_lengths_in_hash_bins(tall, dtype):
+    """Entries and columns of B at the edges of a CTA's windows and chunks with
+    hash look-ups (no column dense), tables in shared memory and, past
+    hash_cta_max products, in scratch.  The longest sum has 300 terms: u = 6e-8
+    in float, so 2e-5 bounds its rounding."""
+    import torch
+    from paper_2303_02471_gb300 import ops
+    rng = np.random.default_rng(29)
+    m = 70001 if tall else 1037
+    lengths = [0, 1, 15, 16, 17, 31, 32, 33, 127, 128, 129, 300]
+    za = np.array([lengths[i % 12] for i in range(720)])
+    zb = np.array([3, 31, 32, 33, 100, 255, 256, 257, 511, 513, 720])
+
+    def matrix(nrows, z):
+        cp = np.concatenate([[0], np.cumsum(z)]).astype(np.int64)
+        rows = np.concatenate([rng.permutation(nrows)[:n] for n in z]).astype(np.int32)
+        return synth.CSC(nrows, len(z), cp, rows, rng.standard_normal(rows.size).astype(dtype))
+    A, B = matrix(m, za), matrix(720, zb)
+    dA, dB = upload(A, dtype), upload(B, dtype)
+    C, plan = ops.spgemm(dA, dB, ops.Config(t=(1 << 63) - 1))
+    bins = plan.info()["bins"]
+    assert bins[13] == 0 and bins[12] > 0 and sum(bins[7:12]) > 0
+    dc = torch.as_tensor(rng.standard_normal(C.nnz).astype(dtype), device="cuda")
+    got = ops.spgemm_backward(plan, dA, dB, C, dc)
+    plan.check()
+    Ch, d = C.to_host(), dc.cpu().numpy()
+    want = oracle.backward(A, B, Ch, d)
+    scale = oracle.backward(A.with_values(np.abs(A.values)), B.with_values(np.abs(B.values)), Ch, np.abs(d))
+    tau = 1e-12 if dtype == np.float64 else 2e-5
+    for g, r, s in zip(got, want, scale):
+        assert np.all(np.abs(g.cpu().numpy().astype(np.float64) - r) <= tau * s)
