@@ -145,8 +145,9 @@ static Geo backward_geometry_t(int bin, int64_t count, int64_t m, int threads, i
     // per window, 1.23 ms now): 256 threads where that
     // keeps as many threads resident as 512, else 512; where the flags live in
     // the per-CTA scratch, the configured size (2^20 rows: double 0.67 ms with
-    // 1024 threads, 1.09 with two CTAs of 512).  The CTA's share of
-    // the SM's shared memory then holds dC[:, j] of the columns it fits.
+    // 1024 threads, 1.09 with two CTAs of 512), and so where the columns are too
+    // few for more CTAs (few_columns).  The CTA's share of the SM's shared
+    // memory then holds dC[:, j] of the columns it fits.
     const size_t bmb = (size_t)W * 8;
     auto shape = [&](int tt, Geo &o) {
         o = g;
@@ -159,7 +160,11 @@ static Geo backward_geometry_t(int bin, int64_t count, int64_t m, int threads, i
     int occ = 0;
     Geo g256, g512;
     const int o256 = threads >= 512 ? shape(256, g256) : 0;
-    if (o256 > 0 && !g256.bm_global) {
+    const int few = few_columns(count, sms, threads);
+    if (o256 > 0 && !g256.bm_global && few) {
+        occ = shape(few, g256);
+        g = g256;
+    } else if (o256 > 0 && !g256.bm_global) {
         const int o512 = shape(512, g512);
         if (o256 * 256 >= o512 * 512) { g = g256; occ = o256; }
         else { g = g512; occ = o512; }
