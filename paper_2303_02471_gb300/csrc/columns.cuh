@@ -314,7 +314,7 @@ __device__ __forceinline__ bool num_dense_column(const TOps<VT> &o, int32_t j, i
     __syncthreads();
     cta_walk<true, VT, kWalkAhead>(o.Acp, o.Arow, o.Aval, o.Brow, o.Bval, o.Bcp[j], o.Bcp[j + 1], w,
                                    [&](int32_t row, VT prod) { atomicAdd(&gacc[bitmap_rank(bm, row)], prod); });
-    cta_bitmap_visit(bm, W, true, s_next, stage, [&](int32_t row) { return o.crow(row); },
+    cta_bitmap_visit(bm, W, true, s_next, stage, nn < W, [&](int32_t row) { return o.crow(row); },
                      [&](int32_t rank, int32_t r) { crow[rank] = r; });
     __syncthreads();
     return true;

@@ -746,43 +746,50 @@ __device__ __forceinline__ int64_t cta_bitmap_prefix(uint2 *bm, int64_t W64, con
 // visit_group(W) chunks of 32 words, the first group by warp index and the
 // next ones from the shared counter *s_next, which must hold
 // visit_group(W) * (number of warps) before a barrier that precedes the call.
-// A warp first lists the group's non-empty words (two thirds of the words of a
-// power-law product's columns are empty), then takes 32 of them at a time, one
-// per lane (R-MAT 2^16 in float 1158 -> 1132 us, R-MAT 2^17's numeric phase
-// 2018 -> 1995 us: the pass was over half of the kernel's instructions, but
-// the adds of the walk bound it).  The ranks of a group are consecutive: a lane writes its word's
-// rows, rank minus the group's first rank being the slot, into the warp's
-// slice of shared memory; the warp then stores the staged slots in order, one
-// per lane, with kVisitUnroll map() look-ups in flight per lane before their
-// stores, so the stores are coalesced and a group waits for few look-up
-// latencies.  A group of more than kVisitStage rows goes through the slice in
-// pieces.  stage: kVisitBytes per warp of shared memory that nothing else uses
-// during the call.  Clears the bits when `clear`.  No barrier inside.
-// Most chunks of 32 words a warp takes per grab (fewer where the warps would
-// otherwise run out of groups).
+// With `list` (columns of fewer rows than words: two thirds of the words of a
+// power-law product's columns are empty) a warp first lists the group's
+// non-empty words, else it takes them all; 32 of them at a time, one per lane.
+// The ranks of a group are consecutive: a lane writes its word's rows, rank
+// minus the group's first rank being the slot, into the warp's slice of shared
+// memory; the warp then stores the staged slots in order, one per lane, with
+// kVisitUnroll map() look-ups in flight per lane before their stores, so the
+// stores are coalesced and a group waits for few look-up latencies.  A group of
+// more rows than the slice holds goes through it in pieces, larger ones without
+// the list (listing the words of all columns cost 10 % of the numeric phase of
+// 2000 columns of 10000 rows out of 30000: 382 us, 345 so).  stage: kVisitBytes
+// per warp of shared memory that nothing else uses during the call.  Clears the
+// bits when `clear`.  No barrier inside.
+// Most chunks of 32 words a warp takes per grab.
 constexpr int kVisitGroup = 4;
-// Rows a warp stages per piece.
-constexpr int kVisitStage = 128;
+// Rows a warp stages per piece, with and without the list.
+constexpr int kVisitListed = 128;
+constexpr int kVisitStage = 160;
 // Look-ups per lane issued before their stores.
 constexpr int kVisitUnroll = 4;
-// Staged rows and the list of words (offsets in the group).
-constexpr int kVisitBytes = kVisitStage * 4 + kVisitGroup * 32;
+// Staged rows, or fewer and the list of words (offsets in the group).
+constexpr int kVisitBytes = kVisitStage * 4;
+static_assert(kVisitListed * 4 + kVisitGroup * 32 <= kVisitBytes, "the list of words follows the staged rows");
 
+// Chunks per grab: one up to four chunks a warp, so that no warp has a grab of
+// four more than another (30 chunks in grabs of three for eight warps: 382 us
+// as above), two up to six (R-MAT 2^16, 47 chunks: numeric phase 918 us with
+// four, 845 with two; R-MAT 2^17, 1881 and 1923), four beyond.
 __device__ __forceinline__ int visit_group(int64_t W) {
-    const int per = ((int)((W + 31) >> 5) * 32) / (int)blockDim.x;  // chunks per warp
-    return per >= kVisitGroup ? kVisitGroup : per < 1 ? 1 : per;
+    const int n = (int)((W + 31) >> 5), nw = (int)blockDim.x >> 5;
+    return n <= 4 * nw ? 1 : n <= 6 * nw ? 2 : kVisitGroup;
 }
 
 template <typename M, typename P>
 __device__ __forceinline__ void cta_bitmap_visit(uint2 *bm, int64_t W64, bool clear, unsigned *s_next,
-                                                 unsigned char *stage, M &&map, P &&put) {
+                                                 unsigned char *stage, bool list, M &&map, P &&put) {
     // m < 2^31, so words, chunks and ranks all fit 32-bit indices
     const int W = (int)W64;
     const int lane = threadIdx.x & 31;
     const int nchunks = (W + 31) >> 5, group = visit_group(W64);
     int32_t *slots = reinterpret_cast<int32_t *>(stage + (threadIdx.x >> 5) * kVisitBytes);
-    unsigned char *words = reinterpret_cast<unsigned char *>(slots + kVisitStage);
+    unsigned char *words = reinterpret_cast<unsigned char *>(slots + kVisitListed);
     const unsigned lt = (1u << lane) - 1u;
+    const int cap = list ? kVisitListed : kVisitStage;
     // stores the slots of relative ranks [from, to), slot 0 holding `from`
     auto flush = [&](int32_t r0, int from, int to) {
         for (int o0 = from; o0 < to; o0 += 32 * kVisitUnroll) {
@@ -803,14 +810,18 @@ __device__ __forceinline__ void cta_bitmap_visit(uint2 *bm, int64_t W64, bool cl
         const int gend = g + group < nchunks ? g + group : nchunks;
         const int w0 = g << 5;
         int n = 0;  // non-empty words
-        for (int c = g; c < gend; ++c) {
-            const int wd = (c << 5) + lane;
-            const bool set = wd < W && bm[wd].x != 0u;
-            const unsigned m = __ballot_sync(0xffffffffu, set);
-            if (set) words[n + __popc(m & lt)] = (unsigned char)(wd - w0);
-            n += __popc(m);
+        if (list) {
+            for (int c = g; c < gend; ++c) {
+                const int wd = (c << 5) + lane;
+                const bool set = wd < W && bm[wd].x != 0u;
+                const unsigned m = __ballot_sync(0xffffffffu, set);
+                if (set) words[n + __popc(m & lt)] = (unsigned char)(wd - w0);
+                n += __popc(m);
+            }
+            __syncwarp();
+        } else {
+            n = (gend << 5) < W ? (gend - g) << 5 : W - w0;
         }
-        __syncwarp();
         // the group's first word exists (g < nchunks); its prefix count is
         // the group's first rank
         const int32_t r0 = (int32_t)bm[w0].y;
@@ -822,7 +833,7 @@ __device__ __forceinline__ void cta_bitmap_visit(uint2 *bm, int64_t W64, bool cl
             int pos = 0;
             int32_t row0 = 0;
             if (i < n) {
-                const int wd = w0 + words[i];
+                const int wd = w0 + (list ? words[i] : i);
                 const uint2 v = bm[wd];
                 if (clear) bm[wd].x = 0u;
                 bits = v.x;
@@ -831,7 +842,7 @@ __device__ __forceinline__ void cta_bitmap_visit(uint2 *bm, int64_t W64, bool cl
             }
             const int end = (int)__reduce_max_sync(0xffffffffu, (unsigned)(pos + __popc(bits)));
             // whole in the slice (uniform over the warp), else in pieces
-            if (end <= flushed + kVisitStage) {
+            if (end <= flushed + cap) {
                 int32_t *to = slots + (pos - flushed);
                 while (bits) {
                     *to++ = row0 + __ffs(bits) - 1;
@@ -839,7 +850,7 @@ __device__ __forceinline__ void cta_bitmap_visit(uint2 *bm, int64_t W64, bool cl
                 }
             } else {
                 for (;;) {
-                    const int lim = flushed + kVisitStage;
+                    const int lim = flushed + cap;
                     while (bits && pos < lim) {
                         slots[pos - flushed] = row0 + __ffs(bits) - 1;
                         bits &= bits - 1u;

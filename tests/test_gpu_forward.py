@@ -649,3 +649,28 @@ def test_few_dense_columns(n, dtype):
     if n <= 20:
         slow = run(ops.Config(cta_threads=256))[2]
         assert times[0] < 0.9 * slow[0] and times[1] < 0.9 * slow[1]
+
+
+@pytest.mark.parametrize("threads", [128, 256, 1024])
+@pytest.mark.parametrize("chunks", [1, 4, 16, 17, 31, 32, 33, 48, 49])
+def test_dense_extraction_densities_and_sizes(chunks, threads):
+    """Columns from one row to all rows (fewer and more rows than flag words,
+    runs longer than a warp's stage), over heights at the edges of the chunks
+    a warp takes at a time."""
+    rng = np.random.default_rng(chunks)
+    m = chunks * 1024 - 3
+    za = np.array([1, 5, m // 32 - 1, m // 32, m // 32 + 2, m // 6, m // 2, m - 1, m])
+    rows = [np.sort(rng.permutation(m)[:z]) for z in za]
+    rows.append(np.arange(min(m, 700)))           # one run
+    rows.append(np.arange(max(0, m - 161), m))    # the last words
+    cp = np.concatenate([[0], np.cumsum([r.size for r in rows])]).astype(np.int64)
+    idx = np.concatenate(rows).astype(np.int32)
+    A = synth.CSC(m, len(rows), cp, idx, rng.standard_normal(idx.size))
+    n = 40  # columns of B: each A column alone, then pairs
+    zb = np.where(np.arange(n) < len(rows), 1, 2)
+    cpb = np.concatenate([[0], np.cumsum(zb)]).astype(np.int64)
+    kb = np.concatenate([[j] if j < len(rows) else rng.permutation(len(rows))[:2] for j in range(n)])
+    B = synth.CSC(len(rows), n, cpb, kb.astype(np.int32), rng.standard_normal(kb.size))
+    C, plan = _run(A, B, t=1, cta_threads=threads)
+    assert plan.info()["bins"][13] == n
+    assert_matches_oracle(C, A, B)
