@@ -753,7 +753,8 @@ spg_status spgemm_backward(spg_plan *P, const spg_csc *A, const spg_csc *B, cons
         for (int b = 1; b < NBINS; ++b) {
             if (!P->host.hist[b]) continue;
             P->bwd_geo[b] = backward_geometry(b, (int64_t)P->host.hist[b], P->mA, P->cfg.cta_threads, P->dev.sms,
-                                              P->dev.smem_optin, (int64_t)P->host.maxnnz[b], P->dtype,
+                                              P->dev.smem_optin, (int64_t)P->host.maxnnz[b],
+                                              (int64_t)(P->host.binnnz[b] / P->host.hist[b]), P->dtype,
                                               P->cfg.table_slots_pct, P->L.scratch_ctas);
         }
         P->bwd_geo_ready = true;

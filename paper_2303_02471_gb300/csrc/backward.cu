@@ -114,7 +114,7 @@ static inline int bwd_cta_threads(int bin, int cfg_threads) {
 
 template <typename VT>
 static Geo backward_geometry_t(int bin, int64_t count, int64_t m, int threads, int sms, size_t smem_optin,
-                               int64_t maxnnz, int slots_pct, int64_t scratch_ctas) {
+                               int64_t maxnnz, int64_t mean_nnz, int slots_pct, int64_t scratch_ctas) {
     Geo g;
     const int64_t W = ceil_div(m, 32);
     if (bin >= BIN_WARP0 && bin < BIN_CTA0) {
@@ -147,7 +147,12 @@ static Geo backward_geometry_t(int bin, int64_t count, int64_t m, int threads, i
     // the per-CTA scratch, the configured size (2^20 rows: double 0.67 ms with
     // 1024 threads, 1.09 with two CTAs of 512), and so where the columns are too
     // few for more CTAs (few_columns).  The CTA's share of the SM's shared
-    // memory then holds dC[:, j] of the columns it fits.
+    // memory then holds dC[:, j] of the columns it fits.  Where a column's dC is
+    // on average more than twice what a 256-thread CTA's share leaves, 512
+    // threads with a larger share win (2000 columns of 20000 products over 100000
+    // rows: double 1125 and 1040 us, float 847 and 732; at 1.1 to 1.5 times they
+    // lose up to 5 %, on R-MAT graphs, whose mean column is light, 20 %), given
+    // more columns than 256-thread CTAs (400 columns: 266 and 296 us).
     const size_t bmb = (size_t)W * 8;
     auto shape = [&](int tt, Geo &o) {
         o = g;
@@ -157,10 +162,15 @@ static Geo backward_geometry_t(int bin, int64_t count, int64_t m, int threads, i
         o.smem = fx + (o.bm_global ? 0 : bmb);
         return occupancy(k_bwd_dense<VT, true>, tt, o.smem);
     };
+    // what the runtime and the kernel's static arrays take
+    constexpr size_t kSmemReserve = 2048;
     int occ = 0;
     Geo g256, g512;
     const int o256 = threads >= 512 ? shape(256, g256) : 0;
-    const int few = few_columns(count, sms, threads);
+    const size_t share256 = smem_optin / 4;
+    const size_t room256 = share256 > g256.smem + kSmemReserve ? share256 - g256.smem - kSmemReserve : 0;
+    const bool long_dc = count > 4 * (int64_t)sms && (size_t)mean_nnz * sizeof(VT) > 2 * room256;
+    const int few = long_dc ? std::min(threads, 512) : few_columns(count, sms, threads);
     if (o256 > 0 && !g256.bm_global && few) {
         occ = shape(few, g256);
         g = g256;
@@ -173,8 +183,6 @@ static Geo backward_geometry_t(int bin, int64_t count, int64_t m, int threads, i
         occ = shape(threads, gc);
         g = gc;
     }
-    // kSmemReserve: what the runtime and the kernel's static arrays take
-    constexpr size_t kSmemReserve = 2048;
     const size_t share = (smem_optin / occ) & ~size_t(127);
     g.cap = 0;
     if (share > g.smem + kSmemReserve)
@@ -188,10 +196,11 @@ static Geo backward_geometry_t(int bin, int64_t count, int64_t m, int threads, i
 }
 
 Geo backward_geometry(int bin, int64_t count, int64_t m, int threads, int sms, size_t smem_optin, int64_t maxnnz,
-                      int dtype, int slots_pct, int64_t scratch_ctas) {
-    return dtype == SPG_F64
-               ? backward_geometry_t<double>(bin, count, m, threads, sms, smem_optin, maxnnz, slots_pct, scratch_ctas)
-               : backward_geometry_t<float>(bin, count, m, threads, sms, smem_optin, maxnnz, slots_pct, scratch_ctas);
+                      int64_t mean_nnz, int dtype, int slots_pct, int64_t scratch_ctas) {
+    return dtype == SPG_F64 ? backward_geometry_t<double>(bin, count, m, threads, sms, smem_optin, maxnnz, mean_nnz,
+                                                          slots_pct, scratch_ctas)
+                            : backward_geometry_t<float>(bin, count, m, threads, sms, smem_optin, maxnnz, mean_nnz,
+                                                         slots_pct, scratch_ctas);
 }
 
 template <typename VT>

@@ -1090,7 +1090,7 @@ cudaError_t launch_backward_bin(const BinTask &t, const Operands &o, const int64
                                 const int32_t *Crow, const void *dC, void *dA, void *dB,
                                 int dtype, const Geo &g, cudaStream_t s);
 Geo backward_geometry(int bin, int64_t count, int64_t m, int threads, int sms, size_t smem_optin,
-                      int64_t maxnnz, int dtype, int slots_pct, int64_t scratch_ctas);
+                      int64_t maxnnz, int64_t mean_nnz, int dtype, int slots_pct, int64_t scratch_ctas);
 
 // Table slots of the global-memory hash bin for a column with Op_j = op in a
 // matrix with m rows (symbolic: keys only, load <= 1/2).

@@ -423,3 +423,31 @@ def test_backward_entry_lengths_in_hash_bins(tall, dtype):
     tau = 1e-12 if dtype == np.float64 else 2e-5
     for g, r, s in zip(got, want, scale):
         assert np.all(np.abs(g.cpu().numpy().astype(np.float64) - r) <= tau * s)
+
+
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+def test_backward_many_columns_of_long_gradients(dtype):
+    """More dense columns than 256-thread CTAs fit the chip, each with a
+    gradient column twice as long as what such a CTA's shared memory leaves (12
+    to 15 thousand rows of 100000), so that CTAs are larger.  The longest sum
+    (dA) has 650 terms: 650 u = 3.9e-5 in float."""
+    import torch
+    from paper_2303_02471_gb300 import ops
+    rng = np.random.default_rng(31)
+    m, k, n = 100000, 3000, 650
+    rows = (np.arange(5)[None, :] * (m // 5) + rng.integers(0, m // 5, (k, 5))).ravel()
+    A = synth.CSC(m, k, np.arange(0, 5 * k + 1, 5), rows.astype(np.int32), rng.standard_normal(5 * k).astype(dtype))
+    B = synth.CSC(k, n, np.arange(0, n * k + 1, k), np.tile(np.arange(k, dtype=np.int32), n),
+                  rng.standard_normal(n * k).astype(dtype))
+    dA, dB = upload(A, dtype), upload(B, dtype)
+    C, plan = ops.spgemm(dA, dB)
+    assert plan.info()["bins"][13] == n
+    dc = torch.as_tensor(rng.standard_normal(C.nnz).astype(dtype), device="cuda")
+    got = ops.spgemm_backward(plan, dA, dB, C, dc)
+    plan.check()
+    Ch, d = C.to_host(), dc.cpu().numpy()
+    want = oracle.backward(A, B, Ch, d)
+    scale = oracle.backward(A.with_values(np.abs(A.values)), B.with_values(np.abs(B.values)), Ch, np.abs(d))
+    tau = 1e-12 if dtype == np.float64 else 650 * 2.0 ** -24
+    for g, r, s in zip(got, want, scale):
+        assert np.all(np.abs(g.cpu().numpy().astype(np.float64) - r) <= tau * s)
