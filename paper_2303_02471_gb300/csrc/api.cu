@@ -202,6 +202,11 @@ struct spg_plan {
     // the larger number of entries of A and B, where the column pointers are
     // known to stay within it (without validation they may point anywhere)
     int64_t entries() const { return cfg.validate ? std::max(nnzA, nnzB) : INT64_MAX; }
+    // bound of nnz(C_j) in a bin for the backward's tables: the largest count,
+    // or (single pass, whose CTA bins count no maximum) what bounds the slots
+    int64_t nnz_bound(int b) const {
+        return host.maxnnz[b] ? (int64_t)host.maxnnz[b] : std::min<int64_t>((int64_t)host.maxop[b], mC);
+    }
     int64_t nonempty_bins() const {
         int64_t n = 0;
         for (int b = 1; b < NBINS; ++b) n += host.hist[b] ? 1 : 0;
@@ -753,7 +758,7 @@ spg_status spgemm_backward(spg_plan *P, const spg_csc *A, const spg_csc *B, cons
         for (int b = 1; b < NBINS; ++b) {
             if (!P->host.hist[b]) continue;
             P->bwd_geo[b] = backward_geometry(b, (int64_t)P->host.hist[b], P->mA, P->cfg.cta_threads, P->dev.sms,
-                                              P->dev.smem_optin, (int64_t)P->host.maxnnz[b],
+                                              P->dev.smem_optin, P->nnz_bound(b),
                                               (int64_t)(P->host.binnnz[b] / P->host.hist[b]), P->dtype,
                                               P->cfg.table_slots_pct, P->L.scratch_ctas);
         }

@@ -100,3 +100,25 @@ def test_operands_of_two_dtypes_are_refused(form, a_is_double):
     plan.check()
     if form != "csr":
         assert_matches_oracle(C, host, host)
+
+
+@pytest.mark.parametrize("acc", ["auto", "hash"])
+@pytest.mark.parametrize("t", [None, 300, (1 << 63) - 1])
+def test_backward_of_a_single_pass_plan_in_every_bin(t, acc):
+    """The single pass counts no largest column per bin: the backward's hash
+    tables are sized by what bounds the columns."""
+    import oracle
+    import torch
+    from paper_2303_02471_gb300 import ops
+    host = synth.rmat(11, seed=6, col_cap=300)
+    A = upload(host)
+    C, plan = ops.spgemm_single_pass(A, A, ops.Config(t=t, small_accumulator=acc))
+    dc = torch.randn(C.nnz, dtype=torch.float64, device="cuda")
+    got = ops.spgemm_backward(plan, A, A, C, dc)
+    plan.check()
+    Ch, d = C.to_host(), dc.cpu().numpy()
+    want = oracle.backward(host, host, Ch, d)
+    Ha = host.with_values(np.abs(host.values))
+    scale = oracle.backward(Ha, Ha, Ch, np.abs(d))
+    for g, r, s in zip(got, want, scale):
+        assert np.all(np.abs(g.cpu().numpy() - r) <= 1e-12 * s)
