@@ -281,8 +281,6 @@ __device__ __forceinline__ bool num_dense_column(const TOps<VT> &o, int32_t j, i
                                                  int64_t W, const uint32_t *keep, const WalkSmem<VT> &w, int64_t *s_warp,
                                                  unsigned *s_next, int32_t *Crow, VT *Cval, AP &&after_prefix,
                                                  int64_t *cnt_out = nullptr) {
-    // the previous user of *s_next finished before the caller's last barrier
-    if (threadIdx.x == 0) *s_next = (blockDim.x >> 5) * visit_group(W);
     // flags kept from the symbolic phase are read straight into the prefix
     // pass; otherwise the walk sets them again
     if (!keep)
@@ -310,11 +308,13 @@ __device__ __forceinline__ bool num_dense_column(const TOps<VT> &o, int32_t j, i
     // has returned (it ends with a barrier): 20 bytes per thread
     static_assert(kVisitBytes <= 32 * (16 + sizeof(float)), "visit staging exceeds the walk scratch");
     unsigned char *stage = reinterpret_cast<unsigned char *>(w.a0);
+    const bool list = nn < W;
+    if (threadIdx.x == 0) *s_next = (blockDim.x >> 5) * visit_group(W, list);
     for (int32_t i = threadIdx.x; i < n32; i += blockDim.x) gacc[i] = VT(0);
     __syncthreads();
     cta_walk<true, VT, kWalkAhead>(o.Acp, o.Arow, o.Aval, o.Brow, o.Bval, o.Bcp[j], o.Bcp[j + 1], w,
                                    [&](int32_t row, VT prod) { atomicAdd(&gacc[bitmap_rank(bm, row)], prod); });
-    cta_bitmap_visit(bm, W, true, s_next, stage, nn < W, [&](int32_t row) { return o.crow(row); },
+    cta_bitmap_visit(bm, W, true, s_next, stage, list, [&](int32_t row) { return o.crow(row); },
                      [&](int32_t rank, int32_t r) { crow[rank] = r; });
     __syncthreads();
     return true;

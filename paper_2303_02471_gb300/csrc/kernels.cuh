@@ -743,9 +743,9 @@ __device__ __forceinline__ int64_t cta_bitmap_prefix(uint2 *bm, int64_t W64, con
 // Writes out the set bits of bm[0..W) in ascending row order: the row at
 // sorted position `rank` of the column is stored by put(rank, map(row))
 // (bm[..].y must hold the prefix counts).  Warps take groups of
-// visit_group(W) chunks of 32 words, the first group by warp index and the
-// next ones from the shared counter *s_next, which must hold
-// visit_group(W) * (number of warps) before a barrier that precedes the call.
+// visit_group(W, list) chunks of 32 words, the first group by warp index and
+// the next ones from the shared counter *s_next, which must hold that times the
+// number of warps before a barrier that precedes the call.
 // With `list` (columns of fewer rows than words: two thirds of the words of a
 // power-law product's columns are empty) a warp first lists the group's
 // non-empty words, else it takes them all; 32 of them at a time, one per lane.
@@ -770,26 +770,33 @@ constexpr int kVisitUnroll = 4;
 constexpr int kVisitBytes = kVisitStage * 4;
 static_assert(kVisitListed * 4 + kVisitGroup * 32 <= kVisitBytes, "the list of words follows the staged rows");
 
-// Chunks per grab: one up to four chunks a warp, so that no warp has a grab of
-// four more than another (30 chunks in grabs of three for eight warps: 382 us
-// as above), two up to six (R-MAT 2^16, 47 chunks: numeric phase 918 us with
-// four, 845 with two; R-MAT 2^17, 1881 and 1923), four beyond.
-__device__ __forceinline__ int visit_group(int64_t W) {
+// Chunks per grab.  Columns taken without the list: one up to four chunks a
+// warp, so that no warp has a grab of four more than another (30 chunks in grabs
+// of three for eight warps: 382 us as above), two up to six (R-MAT 2^16, 47
+// chunks: numeric phase 918 us with four, 845 with two; R-MAT 2^17, 1881 and
+// 1923), four beyond.  With the list a grab's own cost counts more than the
+// balance: the smallest grab that gives each warp one up to two chunks a warp,
+// four beyond (a batch of 12000 columns of 600 rows out of 40000, 40 chunks for
+// 16 warps: 574 us, 617 with grabs of one).
+__device__ __forceinline__ int visit_group(int64_t W, bool list) {
     const int n = (int)((W + 31) >> 5), nw = (int)blockDim.x >> 5;
+    if (list) return n <= 2 * nw ? (n + nw - 1) / nw : kVisitGroup;
     return n <= 4 * nw ? 1 : n <= 6 * nw ? 2 : kVisitGroup;
 }
 
-template <typename M, typename P>
-__device__ __forceinline__ void cta_bitmap_visit(uint2 *bm, int64_t W64, bool clear, unsigned *s_next,
-                                                 unsigned char *stage, bool list, M &&map, P &&put) {
+// One body for each form: the choice inside the loops cost the row-wise product
+// of two random matrices of 60001 rows 1 % (488 against 484 us).
+template <bool list, typename M, typename P>
+__device__ __forceinline__ void cta_bitmap_visit_as(uint2 *bm, int64_t W64, bool clear, unsigned *s_next,
+                                                    unsigned char *stage, M &&map, P &&put) {
     // m < 2^31, so words, chunks and ranks all fit 32-bit indices
     const int W = (int)W64;
     const int lane = threadIdx.x & 31;
-    const int nchunks = (W + 31) >> 5, group = visit_group(W64);
+    const int nchunks = (W + 31) >> 5, group = visit_group(W64, list);
     int32_t *slots = reinterpret_cast<int32_t *>(stage + (threadIdx.x >> 5) * kVisitBytes);
-    unsigned char *words = reinterpret_cast<unsigned char *>(slots + kVisitListed);
+    [[maybe_unused]] unsigned char *words = reinterpret_cast<unsigned char *>(slots + kVisitListed);
     const unsigned lt = (1u << lane) - 1u;
-    const int cap = list ? kVisitListed : kVisitStage;
+    constexpr int cap = list ? kVisitListed : kVisitStage;
     // stores the slots of relative ranks [from, to), slot 0 holding `from`
     auto flush = [&](int32_t r0, int from, int to) {
         for (int o0 = from; o0 < to; o0 += 32 * kVisitUnroll) {
@@ -809,8 +816,8 @@ __device__ __forceinline__ void cta_bitmap_visit(uint2 *bm, int64_t W64, bool cl
     for (int g = (threadIdx.x >> 5) * group; g < nchunks;) {
         const int gend = g + group < nchunks ? g + group : nchunks;
         const int w0 = g << 5;
-        int n = 0;  // non-empty words
-        if (list) {
+        int n = 0;  // non-empty words, or all
+        if constexpr (list) {
             for (int c = g; c < gend; ++c) {
                 const int wd = (c << 5) + lane;
                 const bool set = wd < W && bm[wd].x != 0u;
@@ -872,6 +879,13 @@ __device__ __forceinline__ void cta_bitmap_visit(uint2 *bm, int64_t W64, bool cl
         if (lane == 0) nc = atomicAdd(s_next, (unsigned)group);
         g = (int)__shfl_sync(0xffffffffu, nc, 0);
     }
+}
+
+template <typename M, typename P>
+__device__ __forceinline__ void cta_bitmap_visit(uint2 *bm, int64_t W64, bool clear, unsigned *s_next,
+                                                 unsigned char *stage, bool list, M &&map, P &&put) {
+    if (list) cta_bitmap_visit_as<true>(bm, W64, clear, s_next, stage, map, put);
+    else cta_bitmap_visit_as<false>(bm, W64, clear, s_next, stage, map, put);
 }
 
 // ------------------------------------------------------- bulk copies
