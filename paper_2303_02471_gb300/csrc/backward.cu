@@ -86,8 +86,9 @@ __global__ void __launch_bounds__(1024, 1) k_bwd_dense(BinTask t, Operands o, co
     const size_t o_bm = o_walk + al16((size_t)blockDim.x * 4);
     uint2 *bm = BSM ? reinterpret_cast<uint2 *>(smem + o_bm)
                     : reinterpret_cast<uint2 *>(t.scratch + (size_t)blockIdx.x * t.scratch_stride);
-    // one CTA of every SM (all CTAs of every fourth SM: 1.40 against 1.24 ms
-    // for R-MAT 2^16)
+    // one CTA of every SM, where the blocks go to the SMs in order (all CTAs of
+    // every fourth SM: 1.40 against 1.24 ms for R-MAT 2^16, the graph the choice
+    // was measured on)
     const bool heavy_end = blockIdx.x < (gridDim.x + 3) / 4;
     VT *s_dc = reinterpret_cast<VT *>(smem + o_bm + (BSM ? (size_t)t.W * 8 : 0));
     for (int64_t i = threadIdx.x; i < t.W; i += blockDim.x) bm[i] = make_uint2(0u, 0u);

@@ -127,7 +127,10 @@ __global__ void __launch_bounds__(1024, 1) k_num_dense(BinTask t, Operands o, co
     const unsigned stage_bytes = (unsigned)(t.W * 4);
     // all CTAs of every fourth SM: their adds to C fill the SM's way to L2,
     // which light columns beside them wait for (one CTA of every SM instead:
-    // product of R-MAT 2^18 6.54 against 6.11 ms)
+    // product of R-MAT 2^18 0.4 ms slower).  That block b runs on SM b mod the
+    // number of SMs, and that this number is a multiple of four, is how the
+    // grid lands on this chip, not a promise: anywhere else the columns are
+    // the same and only this gain is lost.
     const bool heavy_end = blockIdx.x % 4 == 0;
     for (int64_t i = threadIdx.x; i < t.W; i += blockDim.x) bm[i] = make_uint2(0u, 0u);
     if (threadIdx.x == 0) {

@@ -103,11 +103,14 @@ __device__ inline void set_error(Ctrl *ctrl, int code, int detail, int64_t index
 // one, the others from the light one.  So a column as heavy as a CTA's whole
 // share (the heaviest of a power-law matrix are) does not start last, and the
 // slices of C in work at a time stay a mixture.  Against the list in column
-// order: backward of R-MAT 2^16 1.46 -> 1.21 ms, product of R-MAT 2^18 6.45 ->
-// 6.11 ms.  Heavy columns on an eighth of the CTAs, or first on a quarter of
-// them with the rest in column order, cost the product of R-MAT 2^18 up to
-// 0.6 ms (more heavy slices of C than L2 holds meet at the end); heaviest
-// first on all CTAs, more.  n: none left.
+// order: backward of R-MAT 2^16 1.46 -> 1.22 ms, product of R-MAT 2^18 6.45 ->
+// 6.0 to 6.2 ms (boxes differ by that much).  Heavy columns on an eighth of the
+// CTAs, or first on a quarter of them with the rest in column order, cost the
+// product of R-MAT 2^18 up to 0.6 ms (more heavy slices of C than L2 holds meet
+// at the end); heaviest first on all CTAs, more.  A quarter is the best of what
+// was tried on these two graphs, not a rule for other distributions of weight;
+// columns of equal weight lose nothing to it (2000 of 20000 products: 384 us,
+// 376 in column order from one counter).  n: none left.
 __device__ inline int64_t next_dense(Ctrl *ctrl, int64_t n, bool heavy_end) {
     if ((int64_t)atomicAdd(&ctrl->work[BIN_DENSE], 1ULL) >= n) return n;
     return heavy_end ? (int64_t)atomicAdd(&ctrl->work[NBINS], 1ULL)

@@ -231,7 +231,7 @@ class Plan:
         self._h = handle
         self._lib_handle = lib_handle  # kept alive while the plan is
         self.workspace = workspace
-        self.slots = None  # single pass: C's columns, until they are copied
+        self.slots = None  # single pass: C's columns, kept with the plan (the library copies from them)
         self.shape = (A.nrows, B.ncols)
         self.dtype = A.dtype
         self.colptr = colptr
